@@ -145,7 +145,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ double s_sum[kMaxRegions];
   __shared__ int s_m;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int qt = blockIdx.x / a.splits, split = blockIdx.x % a.splits;
   const int hk = blockIdx.y, b = blockIdx.z;
 
@@ -275,33 +276,34 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     } else if (warp == 1) {
       // ================================================ MMA issuer
-      if (lane == 0) {
-        bool ok = mbar_wait(bar(DB_Q), 0, abort_flag, a.status, b);
+      // (the whole warp, converged; its elected lane issues: see mma_ss)
+      const uint32_t el = elect_one();
+      const int un = __shfl_sync(0xffffffffu, n, 0);
+      const uint32_t ub = __shfl_sync(0xffffffffu, tbase, 0);
+      bool ok = __all_sync(0xffffffffu, mbar_wait(bar(DB_Q), 0, abort_flag, a.status, b));
+      tc_fence_after();
+      const MatDesc dQ = sdesc_sw128(sbase + L::kQ, 16, 1024);
+      const MatDesc dK = sdesc_sw128(sbase + L::kK, 16, kGroupStride);
+      for (int j = 0; ok && j < un; ++j) {
+        const int st = j % NS, buf = j & 1;
+        ok = mbar_wait(bar(DB_KFULL + st), (j / NS) & 1, abort_flag, a.status, b);
+        if (ok && j >= 2) ok = mbar_wait(bar(DB_SFREE + buf), ((j >> 1) - 1) & 1, abort_flag, a.status, b);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
         tc_fence_after();
-        const uint64_t dQ = sdesc_sw128(sbase + L::kQ, 16, 1024);
-        const uint64_t dK = sdesc_sw128(sbase + L::kK, 16, kGroupStride);
-        for (int j = 0; ok && j < n; ++j) {
-          const int st = j % NS, buf = j & 1;
-          ok = mbar_wait(bar(DB_KFULL + st), (j / NS) & 1, abort_flag, a.status, b);
-          if (ok && j >= 2) ok = mbar_wait(bar(DB_SFREE + buf), ((j >> 1) - 1) & 1, abort_flag, a.status, b);
-          if (!ok) break;
-          tc_fence_after();
-          // K_B's tile follows K_A's with the same 8-row group stride, so
-          // one 256-row operand covers both: S_A in columns 0..127 of the
-          // buffer, S_B in 128..255
-          const uint32_t tS = tbase + buf * 256;
-          const uint64_t dk = dK + (uint64_t)((st * 2 * L::kTile) >> 4);
+        // K_B's tile follows K_A's with the same 8-row group stride, so
+        // one 256-row operand covers both: S_A in columns 0..127 of the
+        // buffer, S_B in 128..255
+        const uint32_t tS = ub + buf * 256;
+        const MatDesc dk = dK.at(st * 2 * L::kTile);
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint64_t qd = dQ + ((kk >> 2) * (BM * 128) + (kk & 3) * 32) / 16;
-            const uint64_t ko = ((kk >> 2) * kPanelOff + (kk & 3) * 32) / 16;
-            mma_ss(tS, qd, dk + ko, IDESC_QK, kk > 0);
-          }
-          mma_commit(bar(DB_SFULL + buf));
-          mma_commit(bar(DB_KEMPTY + st));
-        }
-        mma_commit(bar(DB_FINAL));
+        for (int kk = 0; kk < D / 16; ++kk)
+          mma_ss(tS, dQ.at((kk >> 2) * (BM * 128) + (kk & 3) * 32),
+                 dk.at((kk >> 2) * kPanelOff + (kk & 3) * 32), IDESC_QK, kk > 0, el);
+        mma_commit(bar(DB_SFULL + buf), el);
+        mma_commit(bar(DB_KEMPTY + st), el);
       }
+      mma_commit(bar(DB_FINAL), el);
     } else {
       // ================================================ compute warps
       // Two warps per TMEM lane quarter, each on 64 of the 128 key columns,

@@ -499,38 +499,62 @@ PIC_DEV void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 PIC_DEV void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 PIC_DEV void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// One lane of a converged warp (1 in that lane, 0 in the others).
+PIC_DEV uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+               : "=r"(e));
+  return e;
+}
+// The MMAs and commits below are called by a whole converged warp and take
+// effect in its elected lane (`el` from elect_one).  The descriptors,
+// addresses and loop counters are then warp-uniform and stay in uniform
+// registers.  Issued from an `if (lane == 0)` branch instead, every MMA first
+// moved its operands there, which beside two busy softmax warps per SMSP took
+// 108 cycles an MMA against the 64 the tensor core needs (M128 N128 K16;
+// 66 in this form, measured with the attention kernel's issue order).  A
+// matrix descriptor is passed as its two halves: an offset only moves the
+// low one.
+struct MatDesc {
+  uint32_t lo, hi;
+  PIC_DEV MatDesc at(uint32_t bytes) const { return MatDesc{lo + (bytes >> 4), hi}; }
+};
 // D(tmem) (+)= A(smem desc) * B(smem desc)
-PIC_DEV void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                    uint32_t accumulate) {
+PIC_DEV void mma_ss(uint32_t d_tmem, MatDesc a, MatDesc b, uint32_t idesc, uint32_t accumulate,
+                    uint32_t el) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+      "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+      "setp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 q, %7, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}\n" ::"r"(d_tmem),
+      "r"(a.lo), "r"(a.hi), "r"(b.lo), "r"(b.hi), "r"(idesc), "r"(accumulate), "r"(el)
       : "memory");
 }
 // D(tmem) (+)= A(tmem) * B(smem desc)
-PIC_DEV void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                    uint32_t accumulate) {
+PIC_DEV void mma_ts(uint32_t d_tmem, uint32_t a_tmem, MatDesc b, uint32_t idesc,
+                    uint32_t accumulate, uint32_t el) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 b;\n\tmov.b64 b, {%2, %3};\n\t"
+      "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\t}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "r"(b.lo), "r"(b.hi), "r"(idesc), "r"(accumulate), "r"(el)
       : "memory");
 }
-// Arrive on `bar` once every tcgen05 op issued so far by this thread is done.
-PIC_DEV void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   bar)
-               : "memory");
+// Arrive on `bar` once every tcgen05 op issued so far by the elected lane is done.
+PIC_DEV void mma_commit(uint32_t bar, uint32_t el) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(bar),
+      "r"(el)
+      : "memory");
 }
 // The same commit, arriving on the barrier at this offset in every CTA of
 // the cluster that `cta_mask` selects.
-PIC_DEV void mma_commit_mc(uint32_t bar, uint16_t cta_mask) {
+PIC_DEV void mma_commit_mc(uint32_t bar, uint16_t cta_mask, uint32_t el) {
   asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-      " [%0], %1;" ::"r"(bar), "h"(cta_mask)
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;\n\t}\n" ::"r"(bar), "h"(cta_mask), "r"(el)
       : "memory");
 }
 
@@ -573,14 +597,11 @@ PIC_DEV void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: 
 
 // Shared-memory matrix descriptor for tcgen05.mma, 128-byte swizzle.
 // start/lbo/sbo in bytes (encoded >> 4); version field 1; layout SWIZZLE_128B.
-PIC_DEV uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
+// The start address sits in the low 14 bits; shared addresses stay below
+// 256 KB, so MatDesc::at never carries out of the field.
+PIC_DEV MatDesc sdesc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  return MatDesc{((saddr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16),
+                 ((sbo >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29)};
 }
 
 // Instruction descriptor, kind::f16 with bf16 A/B and fp32 D.

@@ -41,11 +41,11 @@ constexpr int NQ = 2;    // query tiles per CTA, sharing every K/V tile
 constexpr int BN = 128;  // keys per KV tile
 constexpr int NSK = 3;   // K ring stages (released after the last QK of a tile)
 constexpr int NSV = 2;   // V ring stages (released after the last PV of a tile)
-constexpr int kThreads = 128 + NQ * 128;  // K producer, MMA, NQ softmax warpgroups, V producer, relay
+constexpr int kThreads = 96 + NQ * 128;  // K producer, MMA, NQ softmax warpgroups, V producer
 // Rotate-on-load adds a warpgroup that rotates the document keys of each K
 // tile (warps 12-15); its roles are warpgroup-aligned so the registers can be
 // redistributed with setmaxnreg: the control warpgroup (K producer, MMA, V
-// producer, relay) and the rotators give registers to the softmax warpgroups.
+// producer) and the rotators give registers to the softmax warpgroups.
 constexpr int kThreadsFused = 512;
 constexpr int kRegLaunchFused = 65536 / kThreadsFused;  // 128 per thread at launch
 constexpr int kRegCtl = 88, kRegRot = 72, kRegSoftmax = 176;
@@ -54,11 +54,11 @@ static_assert(128 * kRegCtl + 128 * kRegRot + 256 * kRegSoftmax <= 128 * 4 * kRe
 template <bool kFused>
 constexpr int threads_of() { return kFused ? kThreadsFused : kThreads; }
 constexpr int kWarpV = 2 + 4 * NQ;        // the V producer warp
-constexpr int kWarpRelay = kWarpV + 1;    // waits on behalf of the MMA issuer
-// Named barriers between the relay warp and the MMA warp (64 threads each);
-// 0 is __syncthreads, 1 and 2 belong to the softmax warpgroups' epilogue.
-constexpr int kNbPv = 3;  // + t: P_t(j-1) and V(j-1) are ready
-constexpr int kNbK = 5;   // K(j) is ready
+// Named barriers on which the four softmax warps of query tile t hand P_t(j)
+// to the MMA warp; 0 is __syncthreads, 1 and 2 belong to the softmax
+// warpgroups' epilogue.
+constexpr int kNbPv = 3;  // + t
+constexpr int kPvThreads = 128 + 32;
 constexpr int kMaxSplits = 32;
 constexpr uint32_t kTmemCols = 512;
 
@@ -86,8 +86,7 @@ enum {
   B_VFULL = B_KEMPTY + NSK,
   B_VEMPTY = B_VFULL + NSV,
   B_SFULL = B_VEMPTY + NSV,  // one per query tile
-  B_PFULL = B_SFULL + NQ,     // one per query tile (one arrival per softmax warp)
-  B_OFINAL = B_PFULL + NQ,
+  B_OFINAL = B_SFULL + NQ,
   B_KROT = B_OFINAL + 1,  // rotate-on-load: this CTA's half of K(j) rotated (one arrival per rotator warp)
   B_KPEER = B_KROT + NSK,  // rotate-on-load: the cluster peer's rotated half of K(j) has landed
   B_EXIT = B_KPEER + NSK,  // rotate-on-load: the peer is done with this CTA's shared memory
@@ -206,10 +205,15 @@ struct PageSrc {
 // tcgen05 MMAs of one thread complete in order, "S_t(j) is ready" implies
 // PV_t(j-1) has finished, so softmax t may rescale O_t right away, and
 // softmax 0 runs while the tensor core works on tile 1 and vice versa.
-// The MMA issuer does no mbarrier wait inside its loop: an mbarrier wait of
-// a thread queues behind the MMAs that thread issued, so each one left the
-// tensor core idle for a while.  A relay warp waits for K(j), V(j-1) and
-// P_t(j-1) in the issuer's order and hands each over on a named barrier.
+// Bound by the chain S -> softmax -> P -> PV of the two tiles and, on long
+// contexts, by the power limit.  The MMA warp runs converged and issues
+// through its elected lane (mma_ss): issued from a lane-0 branch that also
+// polled the abort flag in shared memory, the 32 MMAs of a key tile took
+// 3360 cycles (tensor core busy 61%) and P always waited for the issuer.
+// P_t goes from the softmax warps to the MMA warp on a named barrier; a warp
+// in between that waited on its behalf (the earlier form) costs the same.
+// 4 x 139k tokens, one layer 3.47 -> 2.95 ms (1380 -> 1630 TFLOP/s); 8 x
+// 16.8k 448 -> 372 us.
 //
 // kFused (rotate-on-load, pic_attend_prefill_fused): the key and value tiles
 // are assembled from the document pool and the cache instead of the stitched
@@ -257,12 +261,11 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + L::kBar + 8 * B_COUNT);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L::kBar + 8 * B_COUNT + 8);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // Warp roles: 0 K producer, 1 MMA issuer, then either 2-9 softmax, 10 V
-  // producer, 11 relay, or (rotate-on-load) 2 V producer, 3 relay, 4-11
-  // softmax, 12-15 rotators.
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  // Warp roles: 0 K producer, 1 MMA issuer, then either 2-9 softmax and 10 V
+  // producer, or (rotate-on-load) 2 V producer, 3 idle, 4-11 softmax, 12-15
+  // rotators.
   constexpr int W_V = kFused ? 2 : kWarpV;
-  constexpr int W_RELAY = kFused ? 3 : kWarpRelay;
   constexpr int W_SM = kFused ? 4 : 2;  // first softmax warp
   constexpr int W_ROT = 12;             // first rotator warp (rotate-on-load)
   // Grid (pair + npairs * split, kv head, request).  CTAs start in linear
@@ -283,8 +286,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
   // the programmatic-launch wait, while that kernel may still be finishing
   if (threadIdx.x == 0) {
     for (int i = 0; i < B_COUNT; ++i)
-      mbar_init(bar(i), ((i >= B_PFULL && i < B_PFULL + NQ) || (i >= B_KROT && i < B_KROT + NSK))
-                            ? 4
+      mbar_init(bar(i), (i >= B_KROT && i < B_KROT + NSK) ? 4
                         : (kFused && i >= B_KEMPTY && i < B_KEMPTY + NSK) ? 2  // both CTAs' QK
                                                                           : 1);
     *abort_flag = 0;
@@ -565,119 +567,81 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
   };
   auto role_issuer = [&]() {
     // ===================================================== MMA issuer
-    // The whole warp takes part in the named barriers; lane 0 issues.  After
-    // an abort both this loop and the relay's run to the end (skipping their
-    // waits and MMAs), so every barrier sync has its arrival.
-    const bool leader = lane == 0;
-    if (leader) mbar_wait(bar(B_Q), 0, abort_flag, p.status, detail);
-    __syncwarp();
-    tc_fence_after();
+    // The whole warp runs this loop, converged, and its elected lane issues
+    // the MMAs and commits (see mma_ss): the loop bounds are made warp-uniform
+    // so that the operands stay in uniform registers.  P_t is handed over by
+    // the softmax warps on a named barrier; after a failed wait (abort) the
+    // loop runs on without waits and MMAs, and the softmax warps meet it at
+    // every barrier, so each barrier still sees all its threads once per tile.
+    const uint32_t el = elect_one();
+    const int un = __shfl_sync(0xffffffffu, n, 0), u_ntile = __shfl_sync(0xffffffffu, ntile, 0);
+    int unt[NQ];
+#pragma unroll
+    for (int t = 0; t < NQ; ++t) unt[t] = __shfl_sync(0xffffffffu, nt[t], 0);
+    const uint32_t ub = __shfl_sync(0xffffffffu, tbase, 0);
+    auto wait = [&](int i, uint32_t parity) -> bool {
+      const bool w = mbar_wait(bar(i), parity, abort_flag, p.status, detail);
+      return __all_sync(0xffffffffu, w);
+    };
+    // K(j) complete in this CTA's ring
+    auto wait_k = [&](int j) -> bool {
+      const uint32_t par = (j / NSK) & 1;
+      if constexpr (kFused) return wait(B_KROT + j % NSK, par) && wait(B_KPEER + j % NSK, par);
+      else return wait(B_KFULL + j % NSK, par);
+    };
     // K(j)'s ring slot is free once every QK reading it has completed -- in
     // rotate-on-load, in both CTAs of the cluster (the peer writes half of it)
     auto release_k = [&](int st) {
-      if constexpr (kFused) mma_commit_mc(bar(B_KEMPTY + st), 0x3);
-      else mma_commit(bar(B_KEMPTY + st));
+      if constexpr (kFused) mma_commit_mc(bar(B_KEMPTY + st), 0x3, el);
+      else mma_commit(bar(B_KEMPTY + st), el);
     };
-    // Matrix descriptors: one base per operand region.  A ring stage, a query
-    // tile or a k-step only moves the start address, which sits in the low 14
-    // bits as address >> 4; shared addresses stay below 256 KB, so adding
-    // (offset >> 4) never carries out of the field.  Built once here, each
-    // MMA costs the issuer an add instead of a full descriptor.
-    const uint64_t dQ = sdesc_sw128(sbase + L::kQ, 16, 1024);
-    const uint64_t dK = sdesc_sw128(sbase + L::kK, 16, kGroupStride);
-    const uint64_t dV = sdesc_sw128(sbase + L::kV, kPanelOff, kGroupStride);
-    for (int j = 0; j <= n; ++j) {
-      bool k_ready = false;
+    // One descriptor base per operand region; a ring stage, a query tile or a
+    // k-step only moves its start address.
+    const MatDesc dQ = sdesc_sw128(sbase + L::kQ, 16, 1024);
+    const MatDesc dK = sdesc_sw128(sbase + L::kK, 16, kGroupStride);
+    const MatDesc dV = sdesc_sw128(sbase + L::kV, kPanelOff, kGroupStride);
+    bool ok = wait(B_Q, 0);
+    for (int j = 0; j <= un; ++j) {
+      // K(j) and V(j-1) are usually there long before P(j-1): waiting for
+      // them first leaves nothing between P's hand-over and the MMAs
+      if (ok && j < un) ok = wait_k(j);
+      if (ok && j >= 1 && j - 1 < unt[0]) ok = wait(B_VFULL + (j - 1) % NSV, ((j - 1) / NSV) & 1);
+      tc_fence_after();
 #pragma unroll
       for (int t = 0; t < NQ; ++t) {
-        if (t >= ntile) break;
-        const uint32_t tS = tbase + t * 128, tO = tbase + 256 + t * 128;
+        if (t >= u_ntile) break;
+        const uint32_t tS = ub + t * 128, tO = ub + 256 + t * 128;
         // O_t += P_t(j-1) V(j-1)
-        if (j >= 1 && j - 1 < nt[t]) {
+        if (j >= 1 && j - 1 < unt[t]) {
           const int pj = j - 1, pst = pj % NSV;
-          named_bar_sync(kNbPv + t, 64);
+          named_bar_sync(kNbPv + t, kPvThreads);
           tc_fence_after();
-          if (leader && !*abort_flag) {
-            const uint64_t dv = dV + (uint64_t)((pst * L::kTile) >> 4);
+          if (ok) {
+            const MatDesc dv = dV.at(pst * L::kTile);
 #pragma unroll
             for (int kk = 0; kk < BN / 16; ++kk)  // one page of 16 keys per MMA
-              mma_ts(tO, tS + kk * 8, dv + (kk * kPageBytes) / 16, IDESC_PV, (pj > 0 || kk > 0));
+              mma_ts(tO, tS + kk * 8, dv.at(kk * kPageBytes), IDESC_PV, (pj > 0 || kk > 0), el);
             // the last tile that reads V(j-1) releases it (tile 1 reads a prefix of tile 0's range)
-            if (t == ntile - 1 || pj >= nt[1]) mma_commit(bar(B_VEMPTY + pst));
+            if (t == u_ntile - 1 || pj >= unt[1]) mma_commit(bar(B_VEMPTY + pst), el);
           }
         }
         // S_t = Q_t K(j)^T
-        if (j < nt[t]) {
+        if (ok && j < unt[t]) {
           const int st = j % NSK;
-          if (!k_ready) {
-            named_bar_sync(kNbK, 64);
-            tc_fence_after();
-            k_ready = true;
-          }
-          if (leader && !*abort_flag) {
-            const uint64_t dk = dK + (uint64_t)((st * L::kTile) >> 4);
-            const uint64_t dq = dQ + (uint64_t)((t * L::kQTile) >> 4);
+          const MatDesc dk = dK.at(st * L::kTile), dq = dQ.at(t * L::kQTile);
 #pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk)
-              mma_ss(tS, dq + ((kk >> 2) * (BM * 128) + (kk & 3) * 32) / 16,
-                     dk + ((kk >> 2) * kPanelOff + (kk & 3) * 32) / 16, IDESC_QK, kk > 0);
-            mma_commit(bar(B_SFULL + t));
-            if (t == ntile - 1 || j >= nt[1]) release_k(st);  // last reader of K(j)
-          }
+          for (int kk = 0; kk < D / 16; ++kk)
+            mma_ss(tS, dq.at((kk >> 2) * (BM * 128) + (kk & 3) * 32),
+                   dk.at((kk >> 2) * kPanelOff + (kk & 3) * 32), IDESC_QK, kk > 0, el);
+          mma_commit(bar(B_SFULL + t), el);
+          if (t == u_ntile - 1 || j >= unt[1]) release_k(st);  // last reader of K(j)
         }
       }
-      if (kFused && j < n && !k_ready) {
-        // A key tile only the cluster peer uses: released once both halves
-        // are in this CTA's ring (its rotators are done with it, the peer's
-        // copy has landed).  The issuer waits itself rather than through the
-        // relay, whose arrivals here would depend on nothing the issuer
-        // does and could run a phase ahead of its syncs.
-        if (leader) {
-          mbar_wait(bar(B_KROT + j % NSK), (j / NSK) & 1, abort_flag, p.status, detail);
-          mbar_wait(bar(B_KPEER + j % NSK), (j / NSK) & 1, abort_flag, p.status, detail);
-          release_k(j % NSK);
-        }
-        __syncwarp();
-      }
+      // a key tile only the cluster peer uses: both halves are in this CTA's
+      // ring (its rotators are done with it, the peer's copy has landed)
+      if (kFused && ok && j < un && j >= unt[0]) release_k(j % NSK);
     }
-    if (leader) mma_commit(bar(B_OFINAL));
-  };
-  auto role_relay = [&]() {
-    // ===================================================== relay for the issuer
-    // Mirrors the issuer's loop: the same conditions, the same order.  Its
-    // arrival on a barrier in iteration j + 1 depends on an MMA the issuer
-    // issues only after its sync on that barrier in iteration j, so the two
-    // never get a phase apart.
-    auto wait_k = [&](int j) {  // K(j) complete in this CTA's ring
-      const uint32_t par = (j / NSK) & 1;
-      if constexpr (kFused) {
-        mbar_wait(bar(B_KROT + j % NSK), par, abort_flag, p.status, detail);
-        mbar_wait(bar(B_KPEER + j % NSK), par, abort_flag, p.status, detail);
-      } else {
-        mbar_wait(bar(B_KFULL + j % NSK), par, abort_flag, p.status, detail);
-      }
-    };
-    for (int j = 0; j <= n; ++j) {
-      bool k_ready = false, v_ready = false;
-#pragma unroll
-      for (int t = 0; t < NQ; ++t) {
-        if (t >= ntile) break;
-        if (j >= 1 && j - 1 < nt[t]) {
-          const int pj = j - 1, pst = pj % NSV;
-          if (!v_ready) {
-            mbar_wait(bar(B_VFULL + pst), (pj / NSV) & 1, abort_flag, p.status, detail);
-            v_ready = true;
-          }
-          mbar_wait(bar(B_PFULL + t), pj & 1, abort_flag, p.status, detail);
-          named_bar_arrive(kNbPv + t, 64);
-        }
-        if (j < nt[t] && !k_ready) {
-          wait_k(j);
-          named_bar_arrive(kNbK, 64);
-          k_ready = true;
-        }
-      }
-    }
+    mma_commit(bar(B_OFINAL), el);
   };
   auto role_rotator = [&]() {
     // ===================================================== rotators (rotate-on-load)
@@ -832,7 +796,8 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     const uint32_t tS = tl + t * 128, tO = tl + 256 + t * 128;
     float m_used = -INFINITY, l = 0.f;
     bool ok = true;
-    for (int j = 0; j < my_n; ++j) {
+    int j_done = 0;  // tiles handed to the issuer
+    for (int j = 0; j < my_n; ++j, ++j_done) {
       const int key0 = (kv_begin + j) * BN;
       if (!__all_sync(0xffffffffu, mbar_wait(bar(B_SFULL + t), j & 1, abort_flag, p.status, detail))) {
         ok = false;
@@ -919,8 +884,10 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_PFULL + t));  // one arrival per warp
+      named_bar_arrive(kNbPv + t, kPvThreads);  // P_t(j) to the MMA warp
     }
+    // after an abort: meet the issuer at the barriers of the remaining tiles
+    for (; j_done < my_n; ++j_done) named_bar_sync(kNbPv + t, kPvThreads);
     // ---- epilogue
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar(B_OFINAL), 0, abort_flag, p.status, detail));
     tc_fence_after();
@@ -994,7 +961,6 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     if constexpr (kGroup == 0) {
       if (warp == 0 || warp == W_V) role_producer();
       else if (warp == 1) role_issuer();
-      else role_relay();
     } else if constexpr (kGroup == 1) {
       role_rotator();
     } else {
@@ -1003,7 +969,6 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
   } else {
     if (warp == 0 || warp == W_V) role_producer();
     else if (warp == 1) role_issuer();
-    else if (warp == W_RELAY) role_relay();
     else role_softmax();
   }
   // Release the dependent launch (the split merge, or the next layer's
@@ -1014,7 +979,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
   __syncthreads();
   if constexpr (kFused) {
     // Leave only when the cluster peer is done too: its last copies into this
-    // CTA's ring have landed (the relay waited for them) and it no longer
+    // CTA's ring have landed (the issuer waited for them) and it no longer
     // reads the copies this CTA sent.  The wait is bounded even after an abort.
     if (threadIdx.x == 0) {
       mbar_arrive_remote(map_to_rank(bar(B_EXIT), cpeer));
@@ -1027,7 +992,9 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     tc_fence_after();
     if (*abort_flag && lane == 0) {
       // make sure no MMA is still running on the TMEM we are about to free
-      mbar_wait(bar(B_OFINAL), 0, abort_flag, p.status, detail);
+      // (bounded by the wait limit alone: the abort flag is already set)
+      volatile int keep_waiting = 0;
+      mbar_wait(bar(B_OFINAL), 0, &keep_waiting, p.status, detail);
     }
     __syncwarp();
     tmem_dealloc(tbase, kTmemCols);
