@@ -200,6 +200,8 @@ def work_of(spec, st):
     L, Hq, Hkv, d = spec.layers, spec.q_heads, spec.kv_heads, spec.head_dim
     lens = [int(x) for x in st.lens]
     doc_tokens = sum(sum(lens[i] for i in docs) for docs in st.docs)
+    # a pool document that several requests list has to be read once
+    pool_read = sum(lens[i] for i in set().union(*st.docs)) if st.docs else 0
     pairs = 0
     query_tokens = 0
     inline_tokens = 0
@@ -221,7 +223,7 @@ def work_of(spec, st):
     row_bytes = Hkv * d * 2
     return {
         "query_tokens": query_tokens,
-        "relocate_bytes": 4 * row_bytes * doc_tokens * L,               # K,V read + write
+        "relocate_bytes": 2 * row_bytes * (pool_read + doc_tokens) * L,  # K,V read + write
         "append_bytes": inline_tokens * (2 * Hq * d * 2 + 4 * row_bytes) * L,
         "attend_flops": 4 * d * Hq * pairs * L,                         # QK^T and PV
         "decode_bytes": sum(2 * row_bytes * (c + 1) for c in ctx) * L,  # K,V of step 0
@@ -560,17 +562,20 @@ def main_gpu(args, rank, world):
                       "tflops": work["attend_flops"] / (per_step["attend"] * 1e9)},
     }
     rows["a2_a3_relocate"]["frac_hbm"] = rows["a2_a3_relocate"]["gbs"] / peaks["hbm_gbs"]
+    # pic_link: one launch, or three when its relocation moves 128 MB or more
+    link_launches = 3 if 8.0 * spec.batch * path.max_ctx * spec.kv_heads * spec.head_dim * L >= 128e6 \
+        else 1
     if link_ms:
         lms = sum(link_ms) / len(link_ms)
         link_bytes = work["relocate_bytes"] + work["append_bytes"] / L
         rows["a1_a4_link"] = {
-            "ms": lms, "launches": 1, "bytes": link_bytes, "gbs": link_bytes / (lms * 1e6),
+            "ms": lms, "launches": link_launches, "bytes": link_bytes, "gbs": link_bytes / (lms * 1e6),
             "frac_hbm": link_bytes / (lms * 1e6) / peaks["hbm_gbs"],
             "note": "pic_link: layout, every layer's relocation and layer 0's inline append in "
-                    "one launch (what the pass runs); rows a1-a4 time the separate calls"}
+                    "one call (what the pass runs); rows a1-a4 time the separate calls"}
     rows["a5_attend"]["frac_bf16"] = rows["a5_attend"]["tflops"] / peaks["bf16_tflops"]
     # kernels of the timed pass: pic_link, the later layers' appends, attention (+ merge)
-    launches = (1 + (L - 1) + rows["a5_attend"]["launches"]) if single else \
+    launches = (link_launches + (L - 1) + rows["a5_attend"]["launches"]) if single else \
         (1 + 1 + L + rows["a5_attend"]["launches"])
 
     # decode (outside the TTFT boundary), same run

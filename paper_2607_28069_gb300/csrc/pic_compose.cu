@@ -31,6 +31,8 @@ struct ComposeArgs {
   const int64_t *doc_start;
   int32_t *doc_offset, *doc_delta, *inline_pos, *ctx_len;
   int64_t *slot_mapping, *tok_map;
+  const int32_t *inline_len;  // nullable; pool_tokens < 0: rows not checked (pic_link checks both)
+  long long pool_tokens;
   int32_t *status;
 };
 
@@ -171,6 +173,8 @@ __global__ void __launch_bounds__(kThreads) compose_kernel(ComposeArgs a) {
         }
         if (t < (long long)s_off[lo] + s_len[lo])
           tm = ((long long)lo << 40) | (s_start[lo] + (t - s_off[lo]));
+        if (a.pool_tokens >= 0 && tm >= 0 && s_start[lo] + (t - s_off[lo]) >= a.pool_tokens)
+          atomicCAS(&s_err, 0, PIC_DEV_BAD_DOC_LEN);
       }
     }
     slots[t] = sl;
@@ -197,24 +201,29 @@ __global__ void __launch_bounds__(kThreads) compose_kernel(ComposeArgs a) {
     }
   }
   __syncthreads();
-  if (tid == 0 && s_err) dev_fail(a.status, s_err, s_err_detail);
-  if (lead && tid == 0) a.ctx_len[b] = s_err ? -1 : (int32_t)ctx;
+  if (tid != 0) return;
+  int fin = s_err;
+  // more inline tokens than prefix, spans and query
+  if (lead && !fin && a.inline_len && min(a.inline_len[b], a.max_inline) > P + n_span + Tq)
+    fin = PIC_DEV_BAD_POSITION;
+  if (fin) dev_fail(a.status, fin, s_err_detail);
+  if (lead) a.ctx_len[b] = fin ? -1 : (int32_t)ctx;
 }
 
 }  // namespace
 }  // namespace pic
 
-extern "C" pic_status_t pic_compose(const pic_geom_t *geom, int32_t batch, int32_t max_docs,
-                                    int32_t n_pool_docs, const int32_t *doc_len,
-                                    const int32_t *doc_base_pos, const int64_t *doc_token_start,
-                                    const int32_t *req_doc_ids,
-                                    const int32_t *req_num_docs, const int32_t *span_len,
-                                    const int32_t *prefix_len,
-                                    const int32_t *query_len, const int32_t *block_table,
-                                    int32_t max_pages, int64_t num_pages, int32_t max_ctx,
-                                    int32_t max_inline, int32_t *doc_offset, int32_t *doc_delta,
-                                    int64_t *slot_mapping, int64_t *tok_map,
-                                    int32_t *inline_pos, int32_t *ctx_len, pic_stream_t stream) {
+pic_status_t pic::compose_layout(const pic_geom_t *geom, int32_t batch, int32_t max_docs,
+                                 int32_t n_pool_docs, const int32_t *doc_len,
+                                 const int32_t *doc_base_pos, const int64_t *doc_token_start,
+                                 const int32_t *req_doc_ids, const int32_t *req_num_docs,
+                                 const int32_t *span_len, const int32_t *prefix_len,
+                                 const int32_t *query_len, const int32_t *block_table,
+                                 int32_t max_pages, int64_t num_pages, int32_t max_ctx,
+                                 int32_t max_inline, int32_t *doc_offset, int32_t *doc_delta,
+                                 int64_t *slot_mapping, int64_t *tok_map, int32_t *inline_pos,
+                                 int32_t *ctx_len, const int32_t *inline_len, int64_t pool_tokens,
+                                 pic_stream_t stream) {
   using namespace pic;
   double theta[kMaxHalfDim];
   pic_status_t st = check_geom(geom, theta);
@@ -256,6 +265,8 @@ extern "C" pic_status_t pic_compose(const pic_geom_t *geom, int32_t batch, int32
   a.ctx_len = ctx_len;
   a.slot_mapping = slot_mapping;
   a.tok_map = tok_map;
+  a.inline_len = inline_len;
+  a.pool_tokens = pool_tokens;
   a.status = status;
   dim3 grid((max_ctx + kSlotsPerCta - 1) / kSlotsPerCta, batch);
   const size_t smem = (size_t)max_docs * (sizeof(long long) + 3 * sizeof(int32_t)) + 16;
@@ -269,4 +280,22 @@ extern "C" pic_status_t pic_compose(const pic_geom_t *geom, int32_t batch, int32
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "pic_compose launch");
   return PIC_OK;
+}
+
+extern "C" pic_status_t pic_compose(const pic_geom_t *geom, int32_t batch, int32_t max_docs,
+                                    int32_t n_pool_docs, const int32_t *doc_len,
+                                    const int32_t *doc_base_pos, const int64_t *doc_token_start,
+                                    const int32_t *req_doc_ids,
+                                    const int32_t *req_num_docs, const int32_t *span_len,
+                                    const int32_t *prefix_len,
+                                    const int32_t *query_len, const int32_t *block_table,
+                                    int32_t max_pages, int64_t num_pages, int32_t max_ctx,
+                                    int32_t max_inline, int32_t *doc_offset, int32_t *doc_delta,
+                                    int64_t *slot_mapping, int64_t *tok_map,
+                                    int32_t *inline_pos, int32_t *ctx_len, pic_stream_t stream) {
+  return pic::compose_layout(geom, batch, max_docs, n_pool_docs, doc_len, doc_base_pos,
+                             doc_token_start, req_doc_ids, req_num_docs, span_len, prefix_len,
+                             query_len, block_table, max_pages, num_pages, max_ctx, max_inline,
+                             doc_offset, doc_delta, slot_mapping, tok_map, inline_pos, ctx_len,
+                             nullptr, -1, stream);
 }

@@ -75,6 +75,46 @@ pic_status_t encode_tmap_3d(CUtensorMap *map, const void *base, uint64_t inner, 
 // stride (the SW128 operand stride) and the two panels 1024 bytes apart.
 pic_status_t encode_tmap_pages128(CUtensorMap *map, const void *base, uint64_t n_page_heads);
 
+// The relocation of pic_link's documents as a launch of its own, after the
+// layout is on the device (relocate_docs_kernel: a shared document is read
+// once, loads by bulk copies), and whether that pays for a relocation that
+// moves up to `bytes`.
+bool link_relocation_apart(double bytes);
+cudaError_t launch_link_relocation(const pic_geom_t *geom, const RopeParams &rp, int batch,
+                                   int max_docs, int n_pool_docs, const void *k_pool,
+                                   const void *v_pool, int64_t pool_tokens,
+                                   const int64_t *doc_token_start, const int32_t *doc_len,
+                                   const int32_t *doc_base_pos, const int32_t *req_doc_ids,
+                                   const int32_t *req_num_docs, const int32_t *prefix_len,
+                                   const int32_t *query_len, const int32_t *doc_offset,
+                                   const int64_t *slot_mapping, int max_ctx, int64_t num_pages,
+                                   void *k_cache, void *v_cache, int layer_begin, int layer_end,
+                                   int32_t *status, cudaStream_t stream);
+
+// pic_compose with pic_link's two further device checks: inline_len (nullable)
+// against the request's inline tokens, and (pool_tokens >= 0) every document
+// row against the pool.
+pic_status_t compose_layout(const pic_geom_t *geom, int32_t batch, int32_t max_docs,
+                            int32_t n_pool_docs, const int32_t *doc_len,
+                            const int32_t *doc_base_pos, const int64_t *doc_token_start,
+                            const int32_t *req_doc_ids, const int32_t *req_num_docs,
+                            const int32_t *span_len, const int32_t *prefix_len,
+                            const int32_t *query_len, const int32_t *block_table,
+                            int32_t max_pages, int64_t num_pages, int32_t max_ctx,
+                            int32_t max_inline, int32_t *doc_offset, int32_t *doc_delta,
+                            int64_t *slot_mapping, int64_t *tok_map, int32_t *inline_pos,
+                            int32_t *ctx_len, const int32_t *inline_len, int64_t pool_tokens,
+                            pic_stream_t stream);
+// pic_append_inline's launch for pic_link, its arguments checked: requests
+// that compose refused as a whole (negative counts) are left alone.
+pic_status_t link_append(const pic_geom_t *geom, const RopeParams &rp, int32_t layer, int32_t batch,
+                         int32_t max_inline, int32_t max_docs, const void *q, const void *k_new,
+                         const void *v_new, const int32_t *inline_pos, const int32_t *inline_len,
+                         const int64_t *slot_mapping, const int32_t *req_num_docs,
+                         const int32_t *prefix_len, const int32_t *query_len, int32_t max_ctx,
+                         int64_t num_pages, void *k_cache, void *v_cache, void *workspace,
+                         pic_stream_t stream);
+
 constexpr int kMaxHalfDim = 64;
 
 // ---------------------------------------------------------- device helpers
@@ -476,6 +516,14 @@ PIC_DEV void tma_load_5d(uint32_t dst, const CUtensorMap *map, int x, int y, int
       "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(v), "r"(bar)
+      : "memory");
+}
+// Untiled bulk copy of `bytes` (a multiple of 16) from global to shared memory,
+// both 16-byte aligned; completes as transaction bytes on `bar`.
+PIC_DEV void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(bar)
       : "memory");
 }
 PIC_DEV void prefetch_tmap(const CUtensorMap *map) {

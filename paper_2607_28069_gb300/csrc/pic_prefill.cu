@@ -1142,6 +1142,8 @@ struct AppendArgs {
   const int32_t *inline_pos, *inline_len;
   const int64_t *slots;          // slot map, or NULL: slots from the block table
   const int32_t *block_table;
+  const int32_t *num_docs, *prefix, *query;  // pic_link's request counts, or NULL
+  int max_docs;
   __nv_bfloat16 *k_cache, *v_cache, *qpack;  // cache pointers already at the layer
   int32_t *status;
 };
@@ -1153,6 +1155,9 @@ __global__ void __launch_bounds__(256) append_kernel(AppendArgs a, RopeParams rp
   const int t = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
   const int tin = min(max(a.inline_len[b], 0), a.max_inline);
   __shared__ float2 cs[HALF];
+  // a request pic_link refused as a whole has no layout to append to
+  if (a.num_docs && (a.num_docs[b] < 0 || a.num_docs[b] > a.max_docs || a.prefix[b] < 0 || a.query[b] < 0))
+    return;
   if (t >= tin) {  // zero the packed query rows of this token slot
     for (int e = tid; e < a.Hkv * a.G * VC; e += blockDim.x) {
       const int hk = e / (a.G * VC), r = e % (a.G * VC), g = r / VC, c = r % VC;
@@ -1481,7 +1486,10 @@ static pic_status_t launch_append(const char *who, const pic_geom_t *geom, const
                                   const int64_t *slot_mapping, const int32_t *block_table,
                                   int32_t max_pages, int32_t max_ctx, int64_t num_pages,
                                   void *k_cache, void *v_cache, void *workspace,
-                                  pic_stream_t stream) {
+                                  pic_stream_t stream, int32_t max_docs = 0,
+                                  const int32_t *num_docs = nullptr,
+                                  const int32_t *prefix_len = nullptr,
+                                  const int32_t *query_len = nullptr) {
   if ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(k_new) |
        reinterpret_cast<uintptr_t>(v_new) | reinterpret_cast<uintptr_t>(k_cache) |
        reinterpret_cast<uintptr_t>(v_cache)) & 15)
@@ -1507,6 +1515,10 @@ static pic_status_t launch_append(const char *who, const pic_geom_t *geom, const
   aa.inline_len = inline_len;
   aa.slots = slot_mapping;
   aa.block_table = block_table;
+  aa.num_docs = num_docs;
+  aa.prefix = prefix_len;
+  aa.query = query_len;
+  aa.max_docs = max_docs;
   aa.k_cache = static_cast<__nv_bfloat16 *>(k_cache) + (size_t)layer * layer_elems;
   aa.v_cache = static_cast<__nv_bfloat16 *>(v_cache) + (size_t)layer * layer_elems;
   aa.qpack = static_cast<__nv_bfloat16 *>(workspace);
@@ -1522,6 +1534,24 @@ static pic_status_t launch_append(const char *who, const pic_geom_t *geom, const
   if (e != cudaSuccess) return cuda_fail(e, "append launch");
   return PIC_OK;
 }
+
+}  // namespace prefill
+
+pic_status_t link_append(const pic_geom_t *geom, const RopeParams &rp, int32_t layer, int32_t batch,
+                         int32_t max_inline, int32_t max_docs, const void *q, const void *k_new,
+                         const void *v_new, const int32_t *inline_pos, const int32_t *inline_len,
+                         const int64_t *slot_mapping, const int32_t *req_num_docs,
+                         const int32_t *prefix_len, const int32_t *query_len, int32_t max_ctx,
+                         int64_t num_pages, void *k_cache, void *v_cache, void *workspace,
+                         pic_stream_t stream) {
+  const prefill::Plan pl = prefill::plan(geom, batch, max_inline, max_ctx, 1);
+  return prefill::launch_append("pic_link", geom, rp, pl, layer, batch, max_inline, q, k_new, v_new,
+                                inline_pos, inline_len, slot_mapping, nullptr, 0, max_ctx, num_pages,
+                                k_cache, v_cache, workspace, stream, max_docs, req_num_docs,
+                                prefix_len, query_len);
+}
+
+namespace prefill {
 
 // The inline projections of a prefill call: all three or none.
 static pic_status_t check_projections(const char *who, const void *q, const void *k_new,

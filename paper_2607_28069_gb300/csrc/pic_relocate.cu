@@ -5,10 +5,10 @@
 //
 // pic_relocate takes the problem as the paper states it: per listed document
 // its pool rows, base position and target position, and the request's block
-// table (relocate_docs_kernel: a CTA per chunk of a document's tokens).
+// table (relocate_docs_kernel: a CTA per slice of a listed document).
 // pic_relocate_mapped takes pic_compose's token and slot maps instead
-// (relocate_kernel, described below); both share the mover of the second
-// half, so for the same placement their caches are bit-identical.
+// (relocate_kernel, described below); both rotate with the same operations,
+// so for the same placement their caches are bit-identical.
 //
 // relocate_kernel: one launch, one CTA per (one or two pages of logical
 // positions, request);
@@ -52,11 +52,13 @@ struct RelocArgs {
   int n_pool_docs, max_pages;
   const int64_t *doc_start;
   const int32_t *doc_len, *doc_base, *ids, *num_docs, *target, *block_table;
+  const int32_t *prefix, *query;  // the link step's (kMapped)
+  bool share;                     // look for documents listed more than once
 };
 
-// Moves the positions a CTA set up (s_src / s_dst / s_doc, the documents'
-// deltas in s_delta) for every layer of [layer_begin, layer_end): the
-// shared second half of both relocation kernels.
+// Moves the positions a CTA of relocate_kernel set up (s_src / s_dst / s_doc,
+// the documents' deltas in s_delta) for every layer of [layer_begin,
+// layer_end).
 template <int D, int kTok, bool kLayerRope>
 __device__ __forceinline__ void move_positions(const RelocArgs &a, const RopeParams &rp, int b,
                                                const long long *s_src, const long long *s_dst,
@@ -126,46 +128,104 @@ __global__ void __launch_bounds__(kThreads) relocate_kernel(RelocArgs a, RopePar
                                       s_cs);
 }
 
-// The per-document form: CTA (slice, k, b) moves the kTok-token chunks
-// slice, slice + S, ... of the k-th listed document of request b (S =
-// gridDim.x): token j of the document (pool row doc_start + j, compiled at
-// base + j) goes to logical position target + j, i.e. to slot
-// block_table[b][(target + j) / 16] * 16 + (target + j) % 16, rotated by
-// delta = target - base.
-template <int D, int kTok, bool kLayerRope>
-__global__ void __launch_bounds__(kThreads) relocate_docs_kernel(RelocArgs a, RopeParams rp) {
+// The per-document form, by pool document: a document that several listed
+// occurrences share (requests of a batch that retrieved the same document, a
+// boundary block repeated in one request) is read once and written to all of
+// them.  CTA (slice, k, b) first finds the other occurrences of its document
+// among the batch's document lists -- up to kMaxShare of them form a group --
+// and then moves every r-th chunk of kTok tokens from its own rank on (r: the
+// group's size; of those, every gridDim.x-th from its slice on) to all r
+// places: token j of the document (pool row doc_start + j, compiled at base +
+// j) goes to logical position target + j of each occurrence, rotated by its
+// delta = target - base.  HBM-bound: 1 + r row transfers a token instead of 2r.
+//
+// The work of a CTA is a list of units (chunk, layer, block of kv heads) of at
+// most 16 KB of K and 16 KB of V, contiguous in the pool: bulk copies bring
+// them into a ring of two stages while the unit before is rotated and stored,
+// so loads stay in flight whatever r is.  Three CTAs an SM.  Measured against
+// a CTA that held 16 tokens in registers and knew one occurrence (four layers
+// unless stated): 8 requests with 16 of 64 1024-token documents 720 -> 510 us
+// (6.3 TB/s of the bytes that must move), 16 with 32 of 64 on 4 kv heads and
+// two layers 740 -> 414, 4 with all 128 of a pool and one layer 869 -> 485;
+// no document shared 275 -> 230 us (6.45 TB/s).  The same sharing with the
+// chunk held in registers (two CTAs an SM) took 564, 473, 566 and 282 us.
+//
+// kMapped (the link step): targets are compose's doc_offset, and slots come
+// from its slot map, -1 wherever its checks refused a position; it has
+// reported the failures itself.
+constexpr int kMaxShare = 8;      // occurrences of a document moved together
+constexpr int kMaxScan = 2048;    // listed documents of a batch up to which a CTA looks for them
+constexpr int kUnit = 8192;       // elements of K (and of V) in a unit
+constexpr int kStageBytes = 2 * kUnit * 2;
+constexpr int kRing = 2;
+constexpr int kRelocSmem = kRing * kStageBytes + 128;
+
+template <int D, int kTok, bool kLayerRope, bool kMapped>
+__global__ void __launch_bounds__(kThreads, 3) relocate_docs_kernel(RelocArgs a, RopeParams rp) {
   pdl_entry();
-  constexpr int HALF = D / 2;
-  const int k = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
-  __shared__ long long s_src[kTok];
-  __shared__ long long s_dst[kTok];
-  __shared__ int s_doc[kTok];
-  __shared__ int s_delta[1];
-  __shared__ float2 s_cs[kLayerRope ? 2 : 1][kTok][HALF];
+  constexpr int HALF = D / 2, KC = D / 16, VC = D / 8;
+  const int k = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, lane = tid & 31, style = rp.style;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t ring = (smem_u32(smem_raw) + 127u) & ~127u;
+  __shared__ uint32_t s_mask[kMaxScan / 32];  // listed documents equal to this one
+  __shared__ int s_tb[kMaxShare], s_tt[kMaxShare];  // request and target position of each
+  __shared__ long long s_row[2][kMaxShare][kTok];   // cache row of head 0 of each token, -1: none
+  __shared__ float2 s_cs[kLayerRope ? 2 : 1][kMaxShare][HALF];
+  __shared__ __align__(8) uint64_t s_bar[kRing];
+  __shared__ int s_abort;
+  if (tid == 0) {
+    for (int i = 0; i < kRing; ++i) mbar_init(smem_u32(&s_bar[i]), 1);
+    s_abort = 0;
+    fence_mbar_init();
+  }
+
+  // ---- this occurrence, and the first 256 listed documents beside it: all
+  // loads independent of one another
+  const int listed = (int)gridDim.z * a.max_docs, own = b * a.max_docs + k;
+  const bool scan = a.share && listed <= kMaxScan;
+  auto target_ok = [&](long long t, int len) {
+    return t >= 0 && (kMapped || t + len <= (long long)a.max_pages * 16);
+  };
+  struct Entry {
+    int id, target;  // id -1: not listed
+  };
+  auto entry = [&](int e) -> Entry {
+    Entry r{-1, -1};
+    if (e < listed) {
+      const int b2 = e / a.max_docs, m2 = a.num_docs[b2];
+      const int id2 = a.ids[e], t2 = a.target[e];
+      const bool bad = kMapped && (a.prefix[b2] < 0 || a.query[b2] < 0);
+      if (m2 <= a.max_docs && e % a.max_docs < m2 && !bad) r = Entry{id2, t2};
+    }
+    return r;
+  };
+  Entry e0{-1, -1};
+  if (scan) e0 = entry(tid);
+  const bool report = !kMapped && tid == 0 && blockIdx.x == 0;
   const int m = a.num_docs[b];
   if (m < 0 || m > a.max_docs) {
-    if (tid == 0 && blockIdx.x == 0 && k == 0) dev_fail(a.status, PIC_DEV_BAD_REQUEST, b);
+    if (report && k == 0) dev_fail(a.status, PIC_DEV_BAD_REQUEST, b);
     return;
   }
   if (k >= m) return;
-  const int id = a.ids[(size_t)b * a.max_docs + k];
+  if (kMapped && (a.prefix[b] < 0 || a.query[b] < 0)) return;
+  const int id = a.ids[own];
+  const long long target = a.target[own];
   if (id < 0 || id >= a.n_pool_docs) {
-    if (tid == 0 && blockIdx.x == 0) dev_fail(a.status, PIC_DEV_BAD_DOC_ID, b);
+    if (report) dev_fail(a.status, PIC_DEV_BAD_DOC_ID, b);
     return;
   }
-  const int n = a.doc_len[id];
+  const int n = a.doc_len[id], base = a.doc_base[id];
   const long long start = a.doc_start[id];
-  if (n <= 0 || start < 0 || start + n > a.pool_tokens) {
-    if (tid == 0 && blockIdx.x == 0) dev_fail(a.status, PIC_DEV_BAD_DOC_LEN, b);
+  if (n <= 0 || (!kMapped && (start < 0 || start + n > a.pool_tokens))) {
+    if (report) dev_fail(a.status, PIC_DEV_BAD_DOC_LEN, b);
     return;
   }
-  const long long target = a.target[(size_t)b * a.max_docs + k];
-  if (target < 0 || target + n > (long long)a.max_pages * 16) {
-    if (tid == 0 && blockIdx.x == 0)
-      dev_fail(a.status, target < 0 ? PIC_DEV_BAD_POSITION : PIC_DEV_BLOCK_TABLE_SHORT, b);
+  if (!target_ok(target, n)) {
+    if (report) dev_fail(a.status, target < 0 ? PIC_DEV_BAD_POSITION : PIC_DEV_BLOCK_TABLE_SHORT, b);
     return;
   }
-  if (blockIdx.x == 0 && tid < 32) {  // targets of two listed documents must not overlap
+  if (!kMapped && blockIdx.x == 0 && tid < 32) {  // targets of two listed documents must not overlap
     bool clash = false;
     for (int k2 = tid; k2 < m; k2 += 32) {
       if (k2 == k) continue;
@@ -177,31 +237,167 @@ __global__ void __launch_bounds__(kThreads) relocate_docs_kernel(RelocArgs a, Ro
     }
     if (__any_sync(0xffffffffu, clash) && tid == 0) dev_fail(a.status, PIC_DEV_BAD_POSITION, b);
   }
-  if (tid == 0) s_delta[0] = (int)(target - a.doc_base[id]);
-  const int32_t *bt = a.block_table + (size_t)b * a.max_pages;
-  const int chunks = (n + kTok - 1) / kTok;
-  for (int c = blockIdx.x; c < chunks; c += gridDim.x) {
-    __syncthreads();  // the previous chunk's maps are no longer read
-    if (tid < kTok) {
-      const int j = c * kTok + tid;
-      long long src = -1, slot = -1;
-      if (j < n) {
-        const long long t = target + j;
-        const int page = bt[t >> 4];
-        if (page < 0 || page >= a.num_pages) {
-          dev_fail(a.status, PIC_DEV_BAD_PAGE, b);
-        } else {
-          src = start + j;
-          slot = (long long)page * 16 + (t & 15);
-        }
-      }
-      s_src[tid] = src;
-      s_dst[tid] = slot;
-      s_doc[tid] = 0;
+
+  // ---- the group: the valid occurrences of the document, in list order
+  int cnt = 1, rank = 0;
+  if (scan) {
+    const int words = (listed + 31) / 32;
+    for (int e = tid; e < words * 32; e += kThreads) {
+      const Entry x = e == tid ? e0 : entry(e);
+      const uint32_t w = __ballot_sync(0xffffffffu, x.id == id && target_ok(x.target, n));
+      if (lane == 0) s_mask[e / 32] = w;
     }
     __syncthreads();
-    move_positions<D, kTok, kLayerRope>(a, rp, b, s_src, s_dst, s_doc, s_delta, 0, 1, s_cs);
+    // every warp: lane l the words 2l and 2l + 1, occurrences before each
+    const uint32_t w0 = 2 * lane < words ? s_mask[2 * lane] : 0u;
+    const uint32_t w1 = 2 * lane + 1 < words ? s_mask[2 * lane + 1] : 0u;
+    int before = __popc(w0) + __popc(w1);
+    const int all = before;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, before, o);
+      if (lane >= o) before += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, before, 31);
+    before -= all;
+    auto rank_of = [&](int e) {  // occurrences before list entry e (e / 32 uniform in the warp)
+      const int w = e / 32;
+      const int base_w = __shfl_sync(0xffffffffu, before + (w & 1 ? __popc(w0) : 0), w / 2);
+      return base_w + __popc(s_mask[w] & ((1u << (e & 31)) - 1u));
+    };
+    rank = rank_of(own);
+    const int first = rank / kMaxShare * kMaxShare;  // the group's first rank
+    for (int e = tid; e < words * 32; e += kThreads) {
+      const int r = rank_of(e) - first;
+      if ((s_mask[e / 32] >> lane & 1u) && r >= 0 && r < kMaxShare) {
+        s_tb[r] = e / a.max_docs;
+        s_tt[r] = e == tid ? e0.target : a.target[e];
+      }
+    }
+    cnt = min(total - first, kMaxShare);
+    rank -= first;
+  } else if (tid == 0) {
+    s_tb[0] = b;
+    s_tt[0] = (int)target;
   }
+  __syncthreads();
+
+  // ---- the units of this CTA: chunk ci of its share, layer, block of heads
+  // tokens j_lo .. j_lo + n_tok - 1 have pool rows (kMapped: maybe not all do)
+  const long long lo = max(0ll, -start), hi = min((long long)n, a.pool_tokens - start);
+  if (lo >= hi) return;
+  const int j_lo = (int)lo, n_tok = (int)(hi - lo);
+  const int chunks = (n_tok + kTok - 1) / kTok;
+  const int c_first = rank + cnt * (int)blockIdx.x, c_step = cnt * (int)gridDim.x;
+  if (c_first >= chunks) return;
+  const int my_chunks = (chunks - c_first + c_step - 1) / c_step;
+  const int hkv = a.hkv, hb = min(hkv, kUnit / (kTok * D)), hblocks = (hkv + hb - 1) / hb;
+  const int layers = a.layer_end - a.layer_begin, per_chunk = layers * hblocks;
+  const long long units = (long long)my_chunks * per_chunk;
+  auto issue = [&](long long u) {  // thread 0: the bulk copies of unit u
+    const int ci = (int)(u / per_chunk), rem = (int)(u % per_chunk);
+    const int layer = a.layer_begin + rem / hblocks, h0 = rem % hblocks * hb, nh = min(hb, hkv - h0);
+    const int t0 = (c_first + ci * c_step) * kTok, nt = min(kTok, n_tok - t0);
+    const size_t src = (((size_t)layer * a.pool_tokens + (start + j_lo + t0)) * hkv + h0) * D;
+    const uint32_t st = ring + (uint32_t)(u % kRing) * kStageBytes, bar = smem_u32(&s_bar[u % kRing]);
+    const uint32_t row = (uint32_t)nh * D * 2;
+    mbar_expect_tx(bar, 2 * nt * row);
+    if (nh == hkv) {  // whole rows: one contiguous piece
+      bulk_load(st, a.k_pool + src, nt * row, bar);
+      bulk_load(st + kUnit * 2, a.v_pool + src, nt * row, bar);
+    } else {
+      for (int i = 0; i < nt; ++i) {
+        bulk_load(st + i * row, a.k_pool + src + (size_t)i * hkv * D, row, bar);
+        bulk_load(st + kUnit * 2 + i * row, a.v_pool + src + (size_t)i * hkv * D, row, bar);
+      }
+    }
+  };
+  if (tid == 0)
+    for (int u = 0; u < min((long long)kRing, units); ++u) issue(u);
+  auto fill_rows = [&](int ci) {  // cache rows of chunk ci's tokens
+    const int t0 = (c_first + ci * c_step) * kTok;
+    for (int e = tid; e < cnt * kTok; e += kThreads) {
+      const int q = e / kTok, i = e % kTok;
+      long long slot = -1;
+      if (t0 + i < n_tok) {
+        const int b2 = s_tb[q];
+        const long long t = (long long)s_tt[q] + j_lo + t0 + i;
+        if (kMapped) {
+          if (t < a.max_ctx) slot = a.slots[(size_t)b2 * a.max_ctx + t];
+          if (slot >= a.num_pages * 16) slot = -1;
+        } else {
+          const int page = a.block_table[(size_t)b2 * a.max_pages + (t >> 4)];
+          if (page < 0 || page >= a.num_pages) dev_fail(a.status, PIC_DEV_BAD_PAGE, b2);
+          else slot = (long long)page * 16 + (t & 15);
+        }
+      }
+      s_row[ci & 1][q][i] = slot < 0 ? -1 : (slot >> 4) * hkv * 16 + (slot & 15);
+    }
+  };
+  auto fill_cs = [&](int layer, int buf) {
+    for (int e = tid; e < cnt * HALF; e += kThreads) {
+      const int q = e / HALF, i = e % HALF, delta = s_tt[q] - base;
+      s_cs[buf][q][i] = kLayerRope ? rope_cos_sin_fast(delta, rope_theta(rp, layer, i))
+                                   : rope_cos_sin(delta, rope_theta(rp, layer, i));
+    }
+  };
+  fill_rows(0);
+  fill_cs(a.layer_begin, 0);
+  __syncthreads();
+
+  const int kc = tid % KC;  // this thread's chunk of 8 pairs, the same in every row
+  const PairChunk pc = pair_chunk(kc, HALF, style);
+  int cur = 0;  // table buffer of the unit's layer (kLayerRope)
+  long long u = 0;
+  bool ok = true;
+  for (int ci = 0; ok && ci < my_chunks; ++ci) {
+    const int nt = min(kTok, n_tok - (c_first + ci * c_step) * kTok);
+    for (int rem = 0; rem < per_chunk; ++rem, ++u) {
+      const int layer = a.layer_begin + rem / hblocks, h0 = rem % hblocks * hb, nh = min(hb, hkv - h0);
+      const uint32_t st = ring + (uint32_t)(u % kRing) * kStageBytes, bar = smem_u32(&s_bar[u % kRing]);
+      // the next chunk's rows and the next layer's table while the copy is in flight
+      if (rem == 0 && ci + 1 < my_chunks) fill_rows(ci + 1);
+      bool next_table = false;
+      if constexpr (kLayerRope) {
+        next_table = layers > 1 && (rem + 1) % hblocks == 0;
+        if (next_table) fill_cs(layer + 1 < a.layer_end ? layer + 1 : a.layer_begin, cur ^ 1);
+      }
+      ok = mbar_wait(bar, (u / kRing) & 1, &s_abort, a.status, b);
+      ok = __syncthreads_and(ok);
+      if (!ok) break;
+      __nv_bfloat16 *kd = a.k_cache + ((size_t)layer * a.num_pages * hkv + h0) * 16 * D;
+      __nv_bfloat16 *vd = a.v_cache + ((size_t)layer * a.num_pages * hkv + h0) * 16 * D;
+      const int nv = nt * nh * VC, nk = nt * nh * KC;
+#pragma unroll 1
+      for (int q = 0; q < cnt; ++q) {
+        const long long *rows = s_row[ci & 1][q];
+        for (int t = tid; t < nv; t += kThreads) {  // values: bit copies
+          const int hr = t / VC, i = hr / nh, h = hr - i * nh;
+          const long long row = rows[i];
+          const uint4 v = lds128(st + kUnit * 2 + t * 16);
+          if (row >= 0) st_global16(vd + (row + h * 16) * D + (t % VC) * 8, v);
+        }
+        float2 cs[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cs[i] = s_cs[cur][q][8 * kc + i];
+        for (int t = tid; t < nk; t += kThreads) {  // keys: rotated by the occurrence's delta
+          const int hr = t / KC, i = hr / nh, h = hr - i * nh;
+          const long long row = rows[i];
+          const uint4 x = lds128(st + (hr * D + pc.off_a) * 2), y = lds128(st + (hr * D + pc.off_b) * 2);
+          if (row >= 0) rotate_store(x, y, kd + (row + h * 16) * D, pc, style, cs);
+        }
+      }
+      fence_proxy_async();  // this thread's reads of the stage precede the next copy into it
+      __syncthreads();
+      if (tid == 0 && u + kRing < units) issue(u + kRing);
+      if (next_table) cur ^= 1;
+    }
+  }
+  if (!ok && tid == 0)  // aborted: let the copies already issued land before the CTA exits
+    for (long long w = u; w < min(units, u + kRing); ++w) {
+      volatile int keep_waiting = 0;
+      mbar_wait(smem_u32(&s_bar[w % kRing]), (w / kRing) & 1, &keep_waiting, a.status, b);
+    }
 }
 
 template <int D, int kTok, bool kLayerRope>
@@ -323,7 +519,83 @@ __device__ __forceinline__ void move_positions(const RelocArgs &a, const RopePar
   }
 }
 
+// Bytes a relocation moves (host estimate: the listed documents at the pool's
+// mean length) from which the search for shared documents pays for itself:
+// it costs a CTA about a microsecond before its first copy (2 requests of 8
+// documents of 512 tokens, 67 MB: 24 us with the search, 19 without; 8 of 16
+// documents of 290, 150 MB: 69 us before, 49 with it).
+constexpr double kShareBytes = 128e6;
+
+// Launch of the per-document form.  Slices per listed document: each CTA
+// walks every slices-th chunk of its share of the document; few documents get
+// more slices (up to one chunk per CTA), so that a small request still fills
+// the GPU (CTAs past a document's last chunk exit).
+template <int D, int kTok, bool kMapped>
+cudaError_t launch_docs_as(const RelocArgs &a, const RopeParams &rp, const dim3 &grid,
+                           cudaStream_t stream) {
+  auto *kernel = rp.layer_theta ? relocate_docs_kernel<D, kTok, true, kMapped>
+                                : relocate_docs_kernel<D, kTok, false, kMapped>;
+  const cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRelocSmem);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(kernel, grid, dim3(kThreads), kRelocSmem, stream, a, rp);
+}
+template <bool kMapped>
+cudaError_t launch_docs(const pic_geom_t *geom, const RelocArgs &a, const RopeParams &rp, int batch,
+                        cudaStream_t stream) {
+  const int row = geom->num_kv_heads * geom->head_dim;
+  const long long docs_total = (long long)batch * a.max_docs;
+  const int slices = (int)std::min<long long>(128, std::max<long long>(16, (8 * 152 + docs_total - 1) / docs_total));
+  const dim3 grid(slices, a.max_docs, batch);
+  if (geom->head_dim == 128)
+    return row >= 1024 ? launch_docs_as<128, 8, kMapped>(a, rp, grid, stream)
+           : row >= 512 ? launch_docs_as<128, 16, kMapped>(a, rp, grid, stream)
+                        : launch_docs_as<128, 32, kMapped>(a, rp, grid, stream);
+  return row >= 1024 ? launch_docs_as<64, 8, kMapped>(a, rp, grid, stream)
+         : row >= 512 ? launch_docs_as<64, 16, kMapped>(a, rp, grid, stream)
+                      : launch_docs_as<64, 32, kMapped>(a, rp, grid, stream);
+}
+
 }  // namespace
+
+cudaError_t launch_link_relocation(const pic_geom_t *geom, const RopeParams &rp, int batch,
+                                   int max_docs, int n_pool_docs, const void *k_pool,
+                                   const void *v_pool, int64_t pool_tokens,
+                                   const int64_t *doc_token_start, const int32_t *doc_len,
+                                   const int32_t *doc_base_pos, const int32_t *req_doc_ids,
+                                   const int32_t *req_num_docs, const int32_t *prefix_len,
+                                   const int32_t *query_len, const int32_t *doc_offset,
+                                   const int64_t *slot_mapping, int max_ctx, int64_t num_pages,
+                                   void *k_cache, void *v_cache, int layer_begin, int layer_end,
+                                   int32_t *status, cudaStream_t stream) {
+  RelocArgs a = {};
+  a.max_docs = max_docs;
+  a.max_ctx = max_ctx;
+  a.hkv = geom->num_kv_heads;
+  a.layer_begin = layer_begin;
+  a.layer_end = layer_end;
+  a.pool_tokens = pool_tokens;
+  a.num_pages = num_pages;
+  a.k_pool = static_cast<const __nv_bfloat16 *>(k_pool);
+  a.v_pool = static_cast<const __nv_bfloat16 *>(v_pool);
+  a.slots = slot_mapping;
+  a.k_cache = static_cast<__nv_bfloat16 *>(k_cache);
+  a.v_cache = static_cast<__nv_bfloat16 *>(v_cache);
+  a.status = status;
+  a.n_pool_docs = n_pool_docs;
+  a.doc_start = doc_token_start;
+  a.doc_len = doc_len;
+  a.doc_base = doc_base_pos;
+  a.ids = req_doc_ids;
+  a.num_docs = req_num_docs;
+  a.target = doc_offset;
+  a.prefix = prefix_len;
+  a.query = query_len;
+  a.share = true;
+  return launch_docs<true>(geom, a, rp, batch, stream);
+}
+
+bool link_relocation_apart(double bytes) { return bytes >= kShareBytes; }
 }  // namespace pic
 
 extern "C" pic_status_t pic_relocate_mapped(const pic_geom_t *geom, int32_t batch,
@@ -448,27 +720,9 @@ extern "C" pic_status_t pic_relocate(const pic_geom_t *geom, int32_t batch, int3
   a.num_docs = req_num_docs;
   a.target = doc_target;
   a.block_table = block_table;
-  const bool wide = geom->num_kv_heads * geom->head_dim >= 1024;
-  // slices per document: each CTA walks every slices-th chunk of its document;
-  // few documents get more slices (up to one chunk per CTA), so that a small
-  // request still fills the GPU (CTAs past a document's last chunk exit)
-  const long long docs_total = (long long)batch * max_docs;
-  const int slices = (int)std::min<long long>(128, std::max<long long>(16, (8 * 152 + docs_total - 1) / docs_total));
-  dim3 grid(slices, max_docs, batch);
-  const dim3 block(kThreads);
-  cudaError_t e;
-  if (geom->head_dim == 128)
-    e = rp.layer_theta
-            ? (wide ? launch_dependent(relocate_docs_kernel<128, 16, true>, grid, block, 0, stream, a, rp)
-                    : launch_dependent(relocate_docs_kernel<128, 32, true>, grid, block, 0, stream, a, rp))
-            : (wide ? launch_dependent(relocate_docs_kernel<128, 16, false>, grid, block, 0, stream, a, rp)
-                    : launch_dependent(relocate_docs_kernel<128, 32, false>, grid, block, 0, stream, a, rp));
-  else
-    e = rp.layer_theta
-            ? (wide ? launch_dependent(relocate_docs_kernel<64, 16, true>, grid, block, 0, stream, a, rp)
-                    : launch_dependent(relocate_docs_kernel<64, 32, true>, grid, block, 0, stream, a, rp))
-            : (wide ? launch_dependent(relocate_docs_kernel<64, 16, false>, grid, block, 0, stream, a, rp)
-                    : launch_dependent(relocate_docs_kernel<64, 32, false>, grid, block, 0, stream, a, rp));
+  a.share = 8.0 * batch * max_docs * ((double)pool_tokens / n_pool_docs) * geom->num_kv_heads *
+                geom->head_dim * (layer_end - layer_begin) >= kShareBytes;
+  cudaError_t e = launch_docs<false>(geom, a, rp, batch, stream);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "pic_relocate launch");
   return PIC_OK;

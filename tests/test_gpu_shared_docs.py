@@ -1,0 +1,109 @@
+"""Documents that several listed occurrences share: pic_relocate reads each once
+and writes it to every occurrence (relocate_docs_kernel), from 128 MB of
+relocation on, and pic_link uses the same kernel.  Both are compared bit for
+bit with pic_relocate_mapped, which moves position by position and knows no
+sharing: groups of one to more than kMaxShare = 8 occurrences, a document
+repeated in one request, head counts that leave a remainder block of heads,
+chunks of 8, 16 and 32 tokens with remainders, both RoPE styles, per-layer
+rotary tables, document lists beyond the 2048 a CTA searches."""
+import pytest
+import torch
+
+from paper_2607_28069_gb300.workloads import custom_spec, generate
+
+pytestmark = pytest.mark.gpu
+
+
+def _spec(name, **kw):
+    return custom_spec(name=name, rope_base=5e5, prefix_len=(3, 70), query_len=19, **kw)
+
+
+CASES = {
+    # name: (spec, rope style, per-layer tables)
+    "pairs": (_spec("pairs", layers=4, q_heads=32, kv_heads=8, head_dim=128, batch=3, pool_docs=9,
+                    docs_per_request=6, doc_len=(100, 700)), 0, False),
+    "groups_over_8": (_spec("groups_over_8", layers=2, q_heads=32, kv_heads=8, head_dim=128,
+                            batch=19, pool_docs=3, docs_per_request=3, doc_len=(1, 333),
+                            span_len=(0, 5)), 1, False),
+    "repeated": (_spec("repeated", layers=5, q_heads=8, kv_heads=4, head_dim=128, batch=2,
+                       pool_docs=4, docs_per_request=7, doc_len=(300, 1700),
+                       fixed_order=(0, 2, 1, 0, 3, 1, 0)), 0, True),
+    "heads_12": (_spec("heads_12", layers=2, q_heads=24, kv_heads=12, head_dim=128, batch=4,
+                       pool_docs=5, docs_per_request=4, doc_len=(200, 900)), 1, False),
+    "d64_h3": (_spec("d64_h3", layers=6, q_heads=6, kv_heads=3, head_dim=64, batch=5, pool_docs=6,
+                     docs_per_request=5, doc_len=(500, 1500)), 0, False),
+    "d64_h16_tables": (_spec("d64_h16_tables", layers=3, q_heads=16, kv_heads=16, head_dim=64,
+                             batch=4, pool_docs=5, docs_per_request=5, doc_len=(150, 800)), 0, True),
+    "beyond_scan": (_spec("beyond_scan", layers=2, q_heads=8, kv_heads=4, head_dim=128, batch=17,
+                          pool_docs=130, docs_per_request=128, doc_len=(1, 30)), 0, False),
+    # one request: nothing shared, but large enough for the three-launch link
+    "one_request": (_spec("one_request", layers=10, q_heads=8, kv_heads=2, head_dim=128, batch=1,
+                          pool_docs=20, docs_per_request=12, doc_len=(300, 1000)), 0, False),
+}
+
+
+def _path(name):
+    from paper_2607_28069_gb300.pipeline import CacheHitPath
+    spec, style, tables = CASES[name]
+    wl = generate(spec, device="cuda", gen_device="cuda")
+    freqs = None
+    if tables:
+        i = torch.arange(spec.head_dim // 2, dtype=torch.float64)
+        freqs = torch.stack([(1e4 if l % 2 else 5e5) ** (-2.0 * i / spec.head_dim)
+                             for l in range(spec.layers)]).cuda()
+    return CacheHitPath(wl, rope_style=style, layer_inv_freq=freqs)
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_shared_documents_bit_identical(cuda_lib, name):
+    import paper_2607_28069_gb300 as pic
+    path = _path(name)
+    spec = path.wl.spec
+    assert 8 * spec.batch * path.max_ctx * spec.kv_heads * spec.head_dim * spec.layers >= 128e6 \
+        or name == "beyond_scan"
+    path.compose()
+    path.relocate_mapped()
+    k_ref, v_ref = path.k_cache.clone(), path.v_cache.clone()
+    path.k_cache.zero_(), path.v_cache.zero_()
+    path.relocate()
+    assert torch.equal(path.k_cache, k_ref) and torch.equal(path.v_cache, v_ref)
+    # pic_link against the three calls: caches, layout, packed queries
+    path.append(0)
+    k_ref, v_ref = path.k_cache.clone(), path.v_cache.clone()
+    packed = path.B * spec.kv_heads * (-(-path.max_inline * spec.q_heads // spec.kv_heads // 128) * 128) \
+        * spec.head_dim * 2
+    ws_ref = path.ws_prefill[:packed].clone()
+    maps = ("doc_offset", "doc_delta", "slot_mapping", "tok_map", "inline_pos", "ctx_len")
+    ref = {m: getattr(path, m).clone() for m in maps}
+    path.k_cache.zero_(), path.v_cache.zero_(), path.ws_prefill.zero_()
+    for m in maps:
+        getattr(path, m).fill_(-7)
+    path.link(0)
+    assert torch.equal(path.k_cache, k_ref) and torch.equal(path.v_cache, v_ref)
+    assert torch.equal(path.ws_prefill[:packed], ws_ref)
+    for m in maps:
+        assert torch.equal(getattr(path, m), ref[m]), m
+    assert pic.pic_device_status() == (0, 0)
+
+
+def test_large_link_refuses_what_the_small_one_does(cuda_lib):
+    """Device checks of the three-launch link: a request with a negative
+    prefix is left alone (nothing of it is written), one with a document id
+    outside the pool is refused as a whole, the others are linked."""
+    import paper_2607_28069_gb300 as pic
+    path = _path("pairs")
+    path.link(0)
+    good = path.k_cache.clone()
+    bt = path.wl.block_table
+    path.k_cache.zero_(), path.v_cache.zero_()
+    path.wl.prefix_len = path.wl.prefix_len.clone()
+    path.wl.prefix_len[0] = -1
+    path.wl.req_doc_ids = path.wl.req_doc_ids.clone()
+    path.wl.req_doc_ids[1, 2] = 99
+    path.link(0)
+    assert pic.pic_device_status()[0] in (1, 3)
+    assert path.ctx_len.tolist()[:2] == [-1, -1]
+    pages = lambda b: bt[b][bt[b] >= 0].long()  # noqa: E731
+    assert not path.k_cache[:, pages(0)].any()
+    assert not path.k_cache[:, pages(1)].any()
+    assert torch.equal(path.k_cache[:, pages(2)], good[:, pages(2)])
