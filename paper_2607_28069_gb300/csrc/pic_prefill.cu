@@ -41,7 +41,7 @@ constexpr int NQ = 2;    // query tiles per CTA, sharing every K/V tile
 constexpr int BN = 128;  // keys per KV tile
 constexpr int NSK = 3;   // K ring stages (released after the last QK of a tile)
 constexpr int NSV = 2;   // V ring stages (released after the last PV of a tile)
-constexpr int kThreads = 96 + NQ * 128;  // K producer, MMA, NQ softmax warpgroups, V producer
+constexpr int kThreads = 128 + NQ * 128;  // K producer, MMA, NQ softmax warpgroups, V producer, ring
 // Rotate-on-load adds a warpgroup that rotates the document keys of each K
 // tile (warps 12-15); its roles are warpgroup-aligned so the registers can be
 // redistributed with setmaxnreg: the control warpgroup (K producer, MMA, V
@@ -54,11 +54,14 @@ static_assert(128 * kRegCtl + 128 * kRegRot + 256 * kRegSoftmax <= 128 * 4 * kRe
 template <bool kFused>
 constexpr int threads_of() { return kFused ? kThreadsFused : kThreads; }
 constexpr int kWarpV = 2 + 4 * NQ;        // the V producer warp
-// Named barriers on which the four softmax warps of query tile t hand P_t(j)
-// to the MMA warp; 0 is __syncthreads, 1 and 2 belong to the softmax
-// warpgroups' epilogue.
-constexpr int kNbPv = 3;  // + t
+constexpr int kWarpRing = kWarpV + 1;     // waits for K and V on the MMA warp's behalf
+// Named barriers; 0 is __syncthreads, 1 and 2 belong to the softmax
+// warpgroups' epilogue.  On 3 + t and 5 + t the four softmax warps of query
+// tile t hand the first kPart keys' columns of P_t(j) and the rest to the MMA
+// warp; on 7 the ring warp meets it once K(j) and V(j-1) are there.
+constexpr int kNbP1 = 3, kNbP2 = 5, kNbRing = 7;
 constexpr int kPvThreads = 128 + 32;
+constexpr int kPart = 64;  // keys of a tile whose P is handed over first
 constexpr int kMaxSplits = 32;
 constexpr uint32_t kTmemCols = 512;
 
@@ -210,10 +213,16 @@ struct PageSrc {
 // through its elected lane (mma_ss): issued from a lane-0 branch that also
 // polled the abort flag in shared memory, the 32 MMAs of a key tile took
 // 3360 cycles (tensor core busy 61%) and P always waited for the issuer.
-// P_t goes from the softmax warps to the MMA warp on a named barrier; a warp
-// in between that waited on its behalf (the earlier form) costs the same.
-// 4 x 139k tokens, one layer 3.47 -> 2.95 ms (1380 -> 1630 TFLOP/s); 8 x
-// 16.8k 448 -> 372 us.
+// One chain sets the period of a tile: S -> softmax -> P -> PV and the next QK
+// of the same query tile, the other tile's MMAs in its gaps.  So the softmax
+// hands P over in two parts, and the first half of PV runs under the second
+// half of the exponentials (clock stamps before: 1424 cycles from S seen to P
+// stored, 1361 from there to the next S seen, 2829 in all with the tensor core
+// busy 2080), and K and V are waited for by a warp of their own (ring).
+// Handing over 32 or 96 of the 128 keys first measured 1-2% slower than 64.
+// Start -> converged issuer -> two parts: one layer of 4 x 139k tokens 3540 ->
+// 3050 -> 2945 us (1.63 PFLOP/s under the power limit, 1.77 at its best), four
+// layers of 8 x 16.8k attention and merge 1914 -> 1613 -> 1500 us.
 //
 // kFused (rotate-on-load, pic_attend_prefill_fused): the key and value tiles
 // are assembled from the document pool and the cache instead of the stitched
@@ -569,26 +578,19 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     // ===================================================== MMA issuer
     // The whole warp runs this loop, converged, and its elected lane issues
     // the MMAs and commits (see mma_ss): the loop bounds are made warp-uniform
-    // so that the operands stay in uniform registers.  P_t is handed over by
-    // the softmax warps on a named barrier; after a failed wait (abort) the
-    // loop runs on without waits and MMAs, and the softmax warps meet it at
-    // every barrier, so each barrier still sees all its threads once per tile.
+    // so that the operands stay in uniform registers.  It touches no shared
+    // memory: with MMAs in flight a satisfied mbarrier wait of this warp takes
+    // about 200 cycles, so the ring warp waits for K and V and meets it on a
+    // named barrier, and P comes on named barriers too.  After an abort
+    // (which the ring warp tells it there) it runs on to the end without
+    // MMAs, and the ring warp and the softmax warps without their waits, so
+    // every barrier sees all its threads once per tile.
     const uint32_t el = elect_one();
     const int un = __shfl_sync(0xffffffffu, n, 0), u_ntile = __shfl_sync(0xffffffffu, ntile, 0);
     int unt[NQ];
 #pragma unroll
     for (int t = 0; t < NQ; ++t) unt[t] = __shfl_sync(0xffffffffu, nt[t], 0);
     const uint32_t ub = __shfl_sync(0xffffffffu, tbase, 0);
-    auto wait = [&](int i, uint32_t parity) -> bool {
-      const bool w = mbar_wait(bar(i), parity, abort_flag, p.status, detail);
-      return __all_sync(0xffffffffu, w);
-    };
-    // K(j) complete in this CTA's ring
-    auto wait_k = [&](int j) -> bool {
-      const uint32_t par = (j / NSK) & 1;
-      if constexpr (kFused) return wait(B_KROT + j % NSK, par) && wait(B_KPEER + j % NSK, par);
-      else return wait(B_KFULL + j % NSK, par);
-    };
     // K(j)'s ring slot is free once every QK reading it has completed -- in
     // rotate-on-load, in both CTAs of the cluster (the peer writes half of it)
     auto release_k = [&](int st) {
@@ -600,33 +602,37 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     const MatDesc dQ = sdesc_sw128(sbase + L::kQ, 16, 1024);
     const MatDesc dK = sdesc_sw128(sbase + L::kK, 16, kGroupStride);
     const MatDesc dV = sdesc_sw128(sbase + L::kV, kPanelOff, kGroupStride);
-    bool ok = wait(B_Q, 0);
     for (int j = 0; j <= un; ++j) {
-      // K(j) and V(j-1) are usually there long before P(j-1): waiting for
-      // them first leaves nothing between P's hand-over and the MMAs
-      if (ok && j < un) ok = wait_k(j);
-      if (ok && j >= 1 && j - 1 < unt[0]) ok = wait(B_VFULL + (j - 1) % NSV, ((j - 1) / NSV) & 1);
+      // K(j) and V(j-1) (and at first Q) are there, or a wait has failed
+      const bool go = !named_bar_or(kNbRing, 64, false);
       tc_fence_after();
 #pragma unroll
       for (int t = 0; t < NQ; ++t) {
         if (t >= u_ntile) break;
         const uint32_t tS = ub + t * 128, tO = ub + 256 + t * 128;
-        // O_t += P_t(j-1) V(j-1)
+        // O_t += P_t(j-1) V(j-1), one page of 16 keys per MMA: the first
+        // kPart keys while the softmax is still at the others
         if (j >= 1 && j - 1 < unt[t]) {
           const int pj = j - 1, pst = pj % NSV;
-          named_bar_sync(kNbPv + t, kPvThreads);
+          const MatDesc dv = dV.at(pst * L::kTile);
+          named_bar_sync(kNbP1 + t, kPvThreads);
           tc_fence_after();
-          if (ok) {
-            const MatDesc dv = dV.at(pst * L::kTile);
+          if (go)
 #pragma unroll
-            for (int kk = 0; kk < BN / 16; ++kk)  // one page of 16 keys per MMA
+            for (int kk = 0; kk < kPart / 16; ++kk)
               mma_ts(tO, tS + kk * 8, dv.at(kk * kPageBytes), IDESC_PV, (pj > 0 || kk > 0), el);
+          named_bar_sync(kNbP2 + t, kPvThreads);
+          tc_fence_after();
+          if (go) {
+#pragma unroll
+            for (int kk = kPart / 16; kk < BN / 16; ++kk)
+              mma_ts(tO, tS + kk * 8, dv.at(kk * kPageBytes), IDESC_PV, 1, el);
             // the last tile that reads V(j-1) releases it (tile 1 reads a prefix of tile 0's range)
             if (t == u_ntile - 1 || pj >= unt[1]) mma_commit(bar(B_VEMPTY + pst), el);
           }
         }
         // S_t = Q_t K(j)^T
-        if (ok && j < unt[t]) {
+        if (go && j < unt[t]) {
           const int st = j % NSK;
           const MatDesc dk = dK.at(st * L::kTile), dq = dQ.at(t * L::kQTile);
 #pragma unroll
@@ -639,9 +645,33 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
       }
       // a key tile only the cluster peer uses: both halves are in this CTA's
       // ring (its rotators are done with it, the peer's copy has landed)
-      if (kFused && ok && j < un && j >= unt[0]) release_k(j % NSK);
+      if (kFused && go && j < un && j >= unt[0]) release_k(j % NSK);
     }
     mma_commit(bar(B_OFINAL), el);
+  };
+  auto role_ring = [&]() {
+    // ===================================================== ring warp
+    // The MMA warp's waits for Q, K(j) (rotate-on-load: both halves) and
+    // V(j-1); it meets the MMA warp once per iteration.
+    bool ok = true;
+    auto wait = [&](int i, uint32_t parity) {
+      if (ok) ok = mbar_wait(bar(i), parity, abort_flag, p.status, detail);
+    };
+    wait(B_Q, 0);
+    for (int j = 0; j <= n; ++j) {
+      if (j < n) {
+        const uint32_t par = (j / NSK) & 1;
+        if constexpr (kFused) {
+          wait(B_KROT + j % NSK, par);
+          wait(B_KPEER + j % NSK, par);
+        } else {
+          wait(B_KFULL + j % NSK, par);
+        }
+      }
+      if (j >= 1 && j - 1 < nt[0]) wait(B_VFULL + (j - 1) % NSV, ((j - 1) / NSV) & 1);
+      ok = __all_sync(0xffffffffu, ok);
+      named_bar_or(kNbRing, 64, !ok);
+    }
   };
   auto role_rotator = [&]() {
     // ===================================================== rotators (rotate-on-load)
@@ -815,18 +845,19 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
       }
       // Exponents against the running maximum m_used.  From the second tile
       // on, a warp whose rows all have one skips the row maximum and
-      // exponentiates against m_used directly; the tile's row sum then bounds
-      // every exponential, and if some row's sum reaches 2^64 (its scores grew
-      // by more than 64 in the log2 domain) the tile is redone the first way:
-      // row maximum, rescale when it grew by more than 2^8, exponentials again.
+      // exponentiates against m_used directly.  Before the first kPart keys'
+      // P is handed over, their sum has to be under 2^63 and the maximum of the
+      // other keys' exponents under 57, which bounds every exponential and the
+      // tile's sum by 2^64; if some row's scores grew past that, nothing has
+      // been handed over yet and the tile is redone the first way: row
+      // maximum, rescale when it grew by more than 2^8, exponentials again.
       // P (bf16) up to 2^64 and the fp32 sums of a few thousand of them stay
       // far inside the range of both.
       float alpha = 1.f;
-      bool resc = false;
       bool need_max = !__all_sync(0xffffffffu, j > 0 && m_used != -INFINITY);
       float l0, l1;
 #pragma unroll 1
-      for (int pass = 0; pass < 2; ++pass) {
+      for (;;) {
         if (need_max) {
           // row max: 4 independent chains of 3-input max
           float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -835,10 +866,22 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
 #pragma unroll
             for (int i = 0; i < 4; ++i) mx[i] = max3f(mx[i], s[c + 2 * i], s[c + 2 * i + 1]);
           const float m_new = fmaxf(m_used, max3f(mx[0], mx[1], fmaxf(mx[2], mx[3])) * p.scale_log2);
-          resc = m_new > m_used + 8.f;
+          const bool resc = m_new > m_used + 8.f;
           if (resc) {
             alpha = ex2(m_used - m_new);
             m_used = m_new;
+          }
+          // O correction: PV_t(j-1) has completed (it precedes QK_t(j) in the MMA order)
+          if (j > 0 && __any_sync(0xffffffffu, resc)) {
+#pragma unroll 1
+            for (int c = 0; c < D / 16; ++c) {
+              float o[16];
+              tmem_ld16(tO + c * 16, reinterpret_cast<uint32_t *>(o));
+              tmem_wait_ld();
+#pragma unroll
+              for (int q = 0; q < 16; ++q) o[q] *= alpha;
+              tmem_st16(tO + c * 16, reinterpret_cast<uint32_t *>(o));
+            }
           }
         }
         const float mref = (m_used == -INFINITY) ? 0.f : m_used;
@@ -846,12 +889,10 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
         // as soon as each 32-key chunk is done (S was read completely above,
         // so the overlap is harmless and the packed values never pile up in
         // registers).  Scaling and the row sum run on packed fp32 pairs (half
-        // the issue slots; the softmax is bound by instruction issue, not by
-        // MUFU).
+        // the issue slots).
         const uint64_t sc2 = f2pack(p.scale_log2, p.scale_log2), nm2 = f2pack(-mref, -mref);
         uint64_t acc[4] = {0, 0, 0, 0};
-#pragma unroll
-        for (int c0 = 0; c0 < BN; c0 += 32) {
+        auto keys32 = [&](int c0) {
           uint32_t pk[16];
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
@@ -862,32 +903,40 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
             pk[q] = pack2(e0, e1);
           }
           tmem_st16(tS + c0 / 2, pk);
+        };
+#pragma unroll
+        for (int c0 = 0; c0 < kPart; c0 += 32) keys32(c0);
+        if (!need_max) {
+          float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+          for (int c = kPart; c < BN; c += 8)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) mx[i] = max3f(mx[i], s[c + 2 * i], s[c + 2 * i + 1]);
+          const float xmax = fmaf(max3f(mx[0], mx[1], fmaxf(mx[2], mx[3])), p.scale_log2, -mref);
+          f2unpack(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), l0, l1);
+          need_max = __any_sync(0xffffffffu, !(l0 + l1 < 0x1p63f) || xmax >= 57.f);
+          if (need_max) continue;
         }
-        acc[0] = add2(add2(acc[0], acc[1]), add2(acc[2], acc[3]));
-        f2unpack(acc[0], l0, l1);
-        if (need_max || !__any_sync(0xffffffffu, !(l0 + l1 < 0x1p64f))) break;
-        need_max = true;
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        named_bar_arrive(kNbP1 + t, kPvThreads);
+#pragma unroll
+        for (int c0 = kPart; c0 < BN; c0 += 32) keys32(c0);
+        f2unpack(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), l0, l1);
+        break;
       }
       l = fmaf(l, alpha, l0 + l1);
-      // O correction: PV_t(j-1) has completed (it precedes QK_t(j) in the MMA order)
-      if (j > 0 && __any_sync(0xffffffffu, resc)) {
-#pragma unroll
-        for (int c = 0; c < D / 32; ++c) {
-          float o[32];
-          tmem_ld32(tO + c * 32, reinterpret_cast<uint32_t *>(o));
-          tmem_wait_ld();
-#pragma unroll
-          for (int q = 0; q < 32; ++q) o[q] *= alpha;
-          tmem_st32(tO + c * 32, reinterpret_cast<uint32_t *>(o));
-        }
-      }
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      named_bar_arrive(kNbPv + t, kPvThreads);  // P_t(j) to the MMA warp
+      named_bar_arrive(kNbP2 + t, kPvThreads);  // the rest of P_t(j)
     }
     // after an abort: meet the issuer at the barriers of the remaining tiles
-    for (; j_done < my_n; ++j_done) named_bar_sync(kNbPv + t, kPvThreads);
+    for (; j_done < my_n; ++j_done) {
+      named_bar_sync(kNbP1 + t, kPvThreads);
+      named_bar_sync(kNbP2 + t, kPvThreads);
+    }
     // ---- epilogue
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar(B_OFINAL), 0, abort_flag, p.status, detail));
     tc_fence_after();
@@ -961,6 +1010,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     if constexpr (kGroup == 0) {
       if (warp == 0 || warp == W_V) role_producer();
       else if (warp == 1) role_issuer();
+      else role_ring();
     } else if constexpr (kGroup == 1) {
       role_rotator();
     } else {
@@ -969,6 +1019,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
   } else {
     if (warp == 0 || warp == W_V) role_producer();
     else if (warp == 1) role_issuer();
+    else if (warp == kWarpRing) role_ring();
     else role_softmax();
   }
   // Release the dependent launch (the split merge, or the next layer's
