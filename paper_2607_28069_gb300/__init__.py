@@ -2,8 +2,9 @@
 
 The functions below carry the names of the C entry points in include/pic.h
 and only marshal arguments (device pointers of torch tensors, sizes, the
-current CUDA stream).  Every step of the path runs in the CUDA kernels of
-libpic.so; if the library is missing, the calls raise -- there is no CPU
+current CUDA stream); those that take tensors do it in _pic_native
+(csrc/binding.cpp).  Every step of the path runs in the CUDA kernels of
+libpic.so; if a library is missing, the calls raise -- there is no CPU
 fallback.
 """
 from __future__ import annotations
@@ -30,6 +31,7 @@ __all__ = [
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_PKG, "libpic.so")
 _lib = None
+_nat = None  # the module _pic_native, loaded with the library
 
 ROPE_HALF = 0
 ROPE_INTERLEAVED = 1
@@ -100,12 +102,13 @@ def lib_path() -> str:
 
 
 def load():
-    """Load libpic.so (raises if it has not been built)."""
-    global _lib
+    """Load libpic.so and _pic_native.so (raises if they have not been built)."""
+    global _lib, _nat
     if _lib is not None:
         return _lib
-    if not os.path.exists(_LIB_PATH):
-        raise RuntimeError(f"{_LIB_PATH} is missing: run __graft_entry__.build() first")
+    for path in (_LIB_PATH, os.path.join(_PKG, "_pic_native.so")):
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: run __graft_entry__.build() first")
     lib = ctypes.CDLL(_LIB_PATH)
     P, I32, I64, SZ, D = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_size_t, ctypes.c_double
     G = ctypes.POINTER(_Geom)
@@ -148,8 +151,17 @@ def load():
         fn.restype = res
         fn.argtypes = args
     del D
+    from . import _pic_native
+    _nat = _pic_native
     _lib = lib
     return lib
+
+
+def _native():
+    """The native part of the binding (loads it at first use)."""
+    if _nat is None:
+        load()
+    return _nat
 
 
 def _check(status: int, what: str):
@@ -162,15 +174,6 @@ def _stream(stream) -> ctypes.c_void_p:
     if stream is None:
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
-
-
-def _ptr_or_pinned(t: torch.Tensor, dtype, name: str):
-    """Like _ptr, for an output that may also live in pinned host memory."""
-    if not t.is_cuda and t.is_pinned():
-        if t.dtype != dtype or not t.is_contiguous():
-            raise ValueError(f"{name} must be a contiguous {dtype} tensor")
-        return ctypes.c_void_p(t.data_ptr())
-    return _ptr(t, dtype, name)
 
 
 def _ptr(t: Optional[torch.Tensor], dtype, name: str, allow_none=False):
@@ -208,17 +211,9 @@ def pic_copy_async(dst: torch.Tensor, src: torch.Tensor, stream=None):
     """Copy the bytes of src into dst (see include/pic.h): each a contiguous
     CUDA tensor of the current device or a pinned CPU tensor, of the same
     size in bytes.  The GPU's own loads and stores move them."""
-    for t, name in ((dst, "dst"), (src, "src")):
-        if not t.is_contiguous():
-            raise ValueError(f"{name} must be contiguous")
-        if not t.is_cuda and not t.is_pinned():
-            raise ValueError(f"{name} must be a CUDA tensor or pinned host memory")
-    nbytes = dst.numel() * dst.element_size()
-    if src.numel() * src.element_size() != nbytes:
-        raise ValueError("dst and src differ in size")
-    st = load().pic_copy_async(ctypes.c_void_p(dst.data_ptr()), ctypes.c_void_p(src.data_ptr()),
-                               nbytes, _stream(stream))
-    _check(st, "pic_copy_async")
+    st = (_nat or _native()).copy_async(dst, src, stream)
+    if st:
+        _check(st, "pic_copy_async")
 
 
 def pic_launch_probe(shapes, stream=None):
@@ -245,20 +240,12 @@ def pic_compose(geom: Geometry, doc_len, doc_base_pos, doc_token_start, req_doc_
                 max_inline: int, doc_offset, doc_delta, slot_mapping, tok_map, inline_pos,
                 ctx_len, stream=None, span_len=None):
     """span_len: int32 [batch][max_docs] post-document inline span lengths, or None."""
-    lib = load()
-    g = geom._c()
-    B, max_docs = req_doc_ids.shape
-    st = lib.pic_compose(
-        ctypes.byref(g), B, max_docs, doc_len.numel(), _ptr(doc_len, i32, "doc_len"),
-        _ptr(doc_base_pos, i32, "doc_base_pos"), _ptr(doc_token_start, i64, "doc_token_start"),
-        _ptr(req_doc_ids, i32, "req_doc_ids"), _ptr(req_num_docs, i32, "req_num_docs"),
-        _ptr(span_len, i32, "span_len", allow_none=True),
-        _ptr(prefix_len, i32, "prefix_len"), _ptr(query_len, i32, "query_len"),
-        _ptr(block_table, i32, "block_table"), block_table.shape[1], num_pages, max_ctx,
-        max_inline, _ptr(doc_offset, i32, "doc_offset"), _ptr(doc_delta, i32, "doc_delta"),
-        _ptr(slot_mapping, i64, "slot_mapping"), _ptr(tok_map, i64, "tok_map"),
-        _ptr(inline_pos, i32, "inline_pos"), _ptr(ctx_len, i32, "ctx_len"), _stream(stream))
-    _check(st, "pic_compose")
+    st = (_nat or _native()).compose(
+        geom, doc_len, doc_base_pos, doc_token_start, req_doc_ids, req_num_docs, span_len,
+        prefix_len, query_len, block_table, num_pages, max_ctx, max_inline, doc_offset, doc_delta,
+        slot_mapping, tok_map, inline_pos, ctx_len, stream)
+    if st:
+        _check(st, "pic_compose")
 
 
 def pic_relocate(geom: Geometry, k_pool, v_pool, doc_token_start, doc_len, doc_base_pos,
@@ -266,37 +253,22 @@ def pic_relocate(geom: Geometry, k_pool, v_pool, doc_token_start, doc_len, doc_b
                  v_cache, layer_begin: int, layer_end: int, stream=None):
     """Per-document relocation: request b's k-th listed document moves from
     its base position to doc_target[b][k] (e.g. pic_compose's doc_offset)."""
-    lib = load()
-    g = geom._c()
-    B, max_docs = req_doc_ids.shape
-    if tuple(doc_target.shape) != (B, max_docs):
-        raise ValueError("doc_target must be [batch][max_docs] like req_doc_ids")
-    st = lib.pic_relocate(
-        ctypes.byref(g), B, max_docs, doc_len.numel(), _ptr(k_pool, bf16, "k_pool"),
-        _ptr(v_pool, bf16, "v_pool"), k_pool.shape[1],
-        _ptr(doc_token_start, i64, "doc_token_start"), _ptr(doc_len, i32, "doc_len"),
-        _ptr(doc_base_pos, i32, "doc_base_pos"), _ptr(req_doc_ids, i32, "req_doc_ids"),
-        _ptr(req_num_docs, i32, "req_num_docs"), _ptr(doc_target, i32, "doc_target"),
-        _ptr(block_table, i32, "block_table"), block_table.shape[1], num_pages,
-        _ptr(k_cache, bf16, "k_cache"), _ptr(v_cache, bf16, "v_cache"), layer_begin, layer_end,
-        _stream(stream))
-    _check(st, "pic_relocate")
+    st = (_nat or _native()).relocate(
+        geom, k_pool, v_pool, doc_token_start, doc_len, doc_base_pos, req_doc_ids, req_num_docs,
+        doc_target, block_table, num_pages, k_cache, v_cache, layer_begin, layer_end, stream)
+    if st:
+        _check(st, "pic_relocate")
 
 
 def pic_relocate_mapped(geom: Geometry, k_pool, v_pool, tok_map, doc_delta, slot_mapping,
                         num_pages: int, k_cache, v_cache, layer_begin: int, layer_end: int,
                         stream=None):
     """Relocation driven by pic_compose's token and slot maps."""
-    lib = load()
-    g = geom._c()
-    B, max_docs = doc_delta.shape
-    st = lib.pic_relocate_mapped(
-        ctypes.byref(g), B, max_docs, _ptr(k_pool, bf16, "k_pool"), _ptr(v_pool, bf16, "v_pool"),
-        k_pool.shape[1], _ptr(tok_map, i64, "tok_map"), _ptr(doc_delta, i32, "doc_delta"),
-        _ptr(slot_mapping, i64, "slot_mapping"), slot_mapping.shape[1], num_pages,
-        _ptr(k_cache, bf16, "k_cache"), _ptr(v_cache, bf16, "v_cache"), layer_begin, layer_end,
-        _stream(stream))
-    _check(st, "pic_relocate_mapped")
+    st = (_nat or _native()).relocate_mapped(
+        geom, k_pool, v_pool, tok_map, doc_delta, slot_mapping, num_pages, k_cache, v_cache,
+        layer_begin, layer_end, stream)
+    if st:
+        _check(st, "pic_relocate_mapped")
 
 
 def pic_link(geom: Geometry, doc_len, doc_base_pos, doc_token_start, req_doc_ids, req_num_docs,
@@ -307,27 +279,13 @@ def pic_link(geom: Geometry, doc_len, doc_base_pos, doc_token_start, req_doc_ids
     """pic_compose + pic_relocate + pic_append_inline (append_layer, or none if < 0)
     in one launch; q/k_new/v_new are the append layer's inline projections;
     span_len as for pic_compose."""
-    lib = load()
-    g = geom._c()
-    B, max_docs = req_doc_ids.shape
-    app = append_layer >= 0
-    st = lib.pic_link(
-        ctypes.byref(g), B, max_docs, doc_len.numel(), _ptr(doc_len, i32, "doc_len"),
-        _ptr(doc_base_pos, i32, "doc_base_pos"), _ptr(doc_token_start, i64, "doc_token_start"),
-        _ptr(req_doc_ids, i32, "req_doc_ids"), _ptr(req_num_docs, i32, "req_num_docs"),
-        _ptr(span_len, i32, "span_len", allow_none=True),
-        _ptr(prefix_len, i32, "prefix_len"), _ptr(query_len, i32, "query_len"),
-        _ptr(block_table, i32, "block_table"), block_table.shape[1], num_pages, max_ctx,
-        max_inline, _ptr(k_pool, bf16, "k_pool"), _ptr(v_pool, bf16, "v_pool"), k_pool.shape[1],
-        layer_begin, layer_end, append_layer, _ptr(q, bf16, "q", allow_none=not app),
-        _ptr(k_new, bf16, "k_new", allow_none=not app), _ptr(v_new, bf16, "v_new", allow_none=not app),
-        _ptr(inline_len, i32, "inline_len", allow_none=not app), _ptr(k_cache, bf16, "k_cache"),
-        _ptr(v_cache, bf16, "v_cache"), _ptr(doc_offset, i32, "doc_offset"),
-        _ptr(doc_delta, i32, "doc_delta"), _ptr(slot_mapping, i64, "slot_mapping"),
-        _ptr(tok_map, i64, "tok_map"), _ptr(inline_pos, i32, "inline_pos"),
-        _ptr(ctx_len, i32, "ctx_len"), _ptr(workspace, torch.uint8, "workspace", allow_none=not app),
-        0 if workspace is None else workspace.numel(), _stream(stream))
-    _check(st, "pic_link")
+    st = (_nat or _native()).link(
+        geom, doc_len, doc_base_pos, doc_token_start, req_doc_ids, req_num_docs, span_len,
+        prefix_len, query_len, block_table, num_pages, max_ctx, max_inline, k_pool, v_pool,
+        layer_begin, layer_end, append_layer, q, k_new, v_new, inline_len, k_cache, v_cache,
+        doc_offset, doc_delta, slot_mapping, tok_map, inline_pos, ctx_len, workspace, stream)
+    if st:
+        _check(st, "pic_link")
 
 
 def pic_prefill_workspace_size(geom: Geometry, batch: int, max_inline: int, max_ctx: int,
@@ -371,25 +329,11 @@ def pic_decode_num_splits(geom: Geometry, batch: int, max_ctx: int, num_splits: 
 
 def pic_append_inline(geom: Geometry, layer: int, q, k_new, v_new, inline_pos, inline_len,
                       slot_mapping, num_pages: int, k_cache, v_cache, workspace, stream=None):
-    lib = load()
-    g = geom._c()
-    B, max_inline = inline_pos.shape
-    st = lib.pic_append_inline(
-        ctypes.byref(g), layer, B, max_inline, _ptr(q, bf16, "q"), _ptr(k_new, bf16, "k_new"),
-        _ptr(v_new, bf16, "v_new"), _ptr(inline_pos, i32, "inline_pos"),
-        _ptr(inline_len, i32, "inline_len"), _ptr(slot_mapping, i64, "slot_mapping"),
-        slot_mapping.shape[1], num_pages, _ptr(k_cache, bf16, "k_cache"),
-        _ptr(v_cache, bf16, "v_cache"), _ptr(workspace, torch.uint8, "workspace"),
-        workspace.numel(), _stream(stream))
-    _check(st, "pic_append_inline")
-
-
-def _projections(q, k_new, v_new):
-    given = [t is not None for t in (q, k_new, v_new)]
-    if any(given) and not all(given):
-        raise ValueError("give q, k_new and v_new together, or none")
-    return (_ptr(q, bf16, "q", allow_none=True), _ptr(k_new, bf16, "k_new", allow_none=True),
-            _ptr(v_new, bf16, "v_new", allow_none=True))
+    st = (_nat or _native()).append_inline(
+        geom, layer, q, k_new, v_new, inline_pos, inline_len, slot_mapping, num_pages, k_cache,
+        v_cache, workspace, stream)
+    if st:
+        _check(st, "pic_append_inline")
 
 
 def pic_attend_prefill(geom: Geometry, layer: int, inline_pos, inline_len, max_ctx: int,
@@ -400,18 +344,11 @@ def pic_attend_prefill(geom: Geometry, layer: int, inline_pos, inline_len, max_c
     un-rotated inline projections) the call appends them itself first;
     without, the workspace must hold this layer's append (pic_append_inline
     or pic_link)."""
-    lib = load()
-    g = geom._c()
-    B, max_inline = inline_pos.shape
-    st = lib.pic_attend_prefill(
-        ctypes.byref(g), layer, B, max_inline, *_projections(q, k_new, v_new),
-        _ptr(inline_pos, i32, "inline_pos"),
-        _ptr(inline_len, i32, "inline_len"), max_ctx, _ptr(block_table, i32, "block_table"),
-        block_table.shape[1], num_pages, _ptr(k_cache, bf16, "k_cache"),
-        _ptr(v_cache, bf16, "v_cache"), _ptr_or_pinned(out, bf16, "out"),
-        _ptr(lse, f32, "lse", allow_none=True), num_splits,
-        _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream))
-    _check(st, "pic_attend_prefill")
+    st = (_nat or _native()).attend_prefill(
+        geom, layer, q, k_new, v_new, inline_pos, inline_len, max_ctx, block_table, num_pages,
+        k_cache, v_cache, out, lse, num_splits, workspace, stream)
+    if st:
+        _check(st, "pic_attend_prefill")
 
 
 def pic_attend_prefill_fused(geom: Geometry, layer: int, inline_pos, inline_len, max_ctx: int,
@@ -421,22 +358,12 @@ def pic_attend_prefill_fused(geom: Geometry, layer: int, inline_pos, inline_len,
     """Rotate-on-load prefill attention: documents read from the pool and
     rotated as they are loaded (tok_map / doc_delta from pic_compose); q,
     k_new, v_new as for pic_attend_prefill."""
-    lib = load()
-    g = geom._c()
-    B, max_inline = inline_pos.shape
-    max_docs = doc_delta.shape[1]
-    if tuple(tok_map.shape) != (B, max_ctx):
-        raise ValueError("tok_map must be [batch][max_ctx]")
-    st = lib.pic_attend_prefill_fused(
-        ctypes.byref(g), layer, B, max_inline, *_projections(q, k_new, v_new),
-        _ptr(inline_pos, i32, "inline_pos"), _ptr(inline_len, i32, "inline_len"), max_ctx,
-        _ptr(block_table, i32, "block_table"), block_table.shape[1], num_pages,
-        _ptr(k_cache, bf16, "k_cache"), _ptr(v_cache, bf16, "v_cache"),
-        _ptr(k_pool, bf16, "k_pool"), _ptr(v_pool, bf16, "v_pool"), k_pool.shape[1], max_docs,
-        _ptr(tok_map, i64, "tok_map"), _ptr(doc_delta, i32, "doc_delta"),
-        _ptr_or_pinned(out, bf16, "out"), _ptr(lse, f32, "lse", allow_none=True), num_splits,
-        _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream))
-    _check(st, "pic_attend_prefill_fused")
+    st = (_nat or _native()).attend_prefill_fused(
+        geom, layer, q, k_new, v_new, inline_pos, inline_len, max_ctx, block_table, num_pages,
+        k_cache, v_cache, k_pool, v_pool, tok_map, doc_delta, out, lse, num_splits, workspace,
+        stream)
+    if st:
+        _check(st, "pic_attend_prefill_fused")
 
 
 def pic_decode_workspace_size(geom: Geometry, batch: int, max_ctx: int, num_splits: int = 0) -> int:
@@ -447,18 +374,11 @@ def pic_decode_workspace_size(geom: Geometry, batch: int, max_ctx: int, num_spli
 def pic_attend_decode(geom: Geometry, layer: int, q, k_new, v_new, pos, block_table,
                       num_pages: int, k_cache, v_cache, out, max_ctx: int, lse=None,
                       num_splits: int = 0, workspace=None, pos_offset: int = 0, stream=None):
-    lib = load()
-    g = geom._c()
-    B = pos.numel()
-    st = lib.pic_attend_decode(
-        ctypes.byref(g), layer, B, _ptr(q, bf16, "q"), _ptr(k_new, bf16, "k_new"),
-        _ptr(v_new, bf16, "v_new"), _ptr(pos, i32, "pos"), pos_offset,
-        _ptr(block_table, i32, "block_table"),
-        block_table.shape[1], num_pages, _ptr(k_cache, bf16, "k_cache"),
-        _ptr(v_cache, bf16, "v_cache"), _ptr(out, bf16, "out"),
-        _ptr(lse, f32, "lse", allow_none=True), max_ctx, num_splits,
-        _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream))
-    _check(st, "pic_attend_decode")
+    st = (_nat or _native()).attend_decode(
+        geom, layer, q, k_new, v_new, pos, pos_offset, block_table, num_pages, k_cache, v_cache,
+        out, lse, max_ctx, num_splits, workspace, stream)
+    if st:
+        _check(st, "pic_attend_decode")
 
 
 def pic_attend_decode_noalloc(geom: Geometry, layer: int, q, k_new, v_new, pos, block_table,
@@ -466,16 +386,11 @@ def pic_attend_decode_noalloc(geom: Geometry, layer: int, q, k_new, v_new, pos, 
                               num_splits: int = 0, pos_offset: int = 0, stream=None):
     """pic_attend_decode without a workspace, for callers that cannot allocate
     while decoding; the scratch is an array inside the library (see pic.h)."""
-    lib = load()
-    g = geom._c()
-    B = pos.numel()
-    st = lib.pic_attend_decode_noalloc(
-        ctypes.byref(g), layer, B, _ptr(q, bf16, "q"), _ptr(k_new, bf16, "k_new"),
-        _ptr(v_new, bf16, "v_new"), _ptr(pos, i32, "pos"), pos_offset,
-        _ptr(block_table, i32, "block_table"), block_table.shape[1], num_pages,
-        _ptr(k_cache, bf16, "k_cache"), _ptr(v_cache, bf16, "v_cache"), _ptr(out, bf16, "out"),
-        _ptr(lse, f32, "lse", allow_none=True), max_ctx, num_splits, _stream(stream))
-    _check(st, "pic_attend_decode_noalloc")
+    st = (_nat or _native()).attend_decode_noalloc(
+        geom, layer, q, k_new, v_new, pos, pos_offset, block_table, num_pages, k_cache, v_cache,
+        out, lse, max_ctx, num_splits, stream)
+    if st:
+        _check(st, "pic_attend_decode_noalloc")
 
 
 def pic_attention_deviation(geom: Geometry, layer: int, inline_pos, inline_len, query_len,
@@ -486,21 +401,11 @@ def pic_attention_deviation(geom: Geometry, layer: int, inline_pos, inline_len, 
     """D_r(A, B) of two stitched key caches (see include/pic.h): fills
     sums [B][R] (float64) and counts [B][R] (int64) for the regions between
     consecutive ``edges``."""
-    lib = load()
-    g = geom._c()
-    B, max_inline = inline_pos.shape
     if max_query_len is None:
         max_query_len = int(query_len.max().item())
-    arr = (ctypes.c_double * len(edges))(*[float(e) for e in edges])
-    st = lib.pic_attention_deviation(
-        ctypes.byref(g), layer, B, max_inline, req_doc_ids.shape[1], slot_mapping.shape[1],
-        num_pages, _ptr(inline_pos, i32, "inline_pos"), _ptr(inline_len, i32, "inline_len"),
-        _ptr(query_len, i32, "query_len"), int(max_query_len), _ptr(req_doc_ids, i32, "req_doc_ids"),
-        _ptr(doc_len, i32, "doc_len"), _ptr(doc_offset, i32, "doc_offset"),
-        _ptr(slot_mapping, i64, "slot_mapping"),
-        _ptr(k_cache_a, bf16, "k_cache_a"), _ptr(k_cache_b, bf16, "k_cache_b"),
-        _ptr(lse_a, f32, "lse_a"), _ptr(lse_b, f32, "lse_b"), ctypes.cast(arr, ctypes.c_void_p),
-        len(edges) - 1,
-        _ptr(workspace, torch.uint8, "workspace"), workspace.numel(),
-        _ptr(sums, torch.float64, "sums"), _ptr(counts, i64, "counts"), _stream(stream))
-    _check(st, "pic_attention_deviation")
+    st = (_nat or _native()).attention_deviation(
+        geom, layer, inline_pos, inline_len, query_len, int(max_query_len), req_doc_ids, doc_len,
+        doc_offset, slot_mapping, num_pages, k_cache_a, k_cache_b, lse_a, lse_b, edges, workspace,
+        sums, counts, stream)
+    if st:
+        _check(st, "pic_attention_deviation")

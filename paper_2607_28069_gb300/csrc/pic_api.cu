@@ -112,8 +112,17 @@ pic_status_t check_geom(const pic_geom_t *g, double *theta) {
   } else {
     if (!(g->rope_base > 1.0) || !std::isfinite(g->rope_base))
       return fail(PIC_ERR_INVALID_ARG, "rope_base must be > 1");
-    for (int i = 0; i < half; ++i)
-      theta[i] = std::pow(g->rope_base, -2.0 * (double)i / (double)g->head_dim);
+    // a model's calls all have the same base: its powers are formed once per
+    // thread and base (2 us a call on a Grace core)
+    static thread_local double memo[kMaxHalfDim], memo_base = 0.0;
+    static thread_local int memo_dim = 0;
+    if (memo_base != g->rope_base || memo_dim != g->head_dim) {
+      for (int i = 0; i < half; ++i)
+        memo[i] = std::pow(g->rope_base, -2.0 * (double)i / (double)g->head_dim);
+      memo_base = g->rope_base;
+      memo_dim = g->head_dim;
+    }
+    for (int i = 0; i < half; ++i) theta[i] = memo[i];
   }
   for (int i = half; i < kMaxHalfDim; ++i) theta[i] = 0.0;
   return PIC_OK;

@@ -8,7 +8,7 @@ from __future__ import annotations
 
 import torch
 
-from . import (Geometry, pic_append_inline, pic_attend_decode, pic_attend_prefill,
+from . import (Geometry, _check, _native, pic_append_inline, pic_attend_decode, pic_attend_prefill,
                pic_attend_prefill_fused, pic_compose, pic_copy_async, pic_decode_workspace_size,
                pic_link, pic_prefill_fused_workspace_size, pic_prefill_plan_splits, pic_relocate,
                pic_relocate_mapped)
@@ -49,6 +49,10 @@ def host_inline_positions(wl: Workload):
 
 
 class CacheHitPath:
+    """Buffers and calls of one workload.  Layer `l` of a tensor with a leading
+    layer dimension goes to the calls as the tuple (tensor, l), which the
+    binding takes for tensor[l] without creating a view of it."""
+
     def __init__(self, wl: Workload, prefill_splits: int = 0, decode_splits: int = 0,
                  with_lse: bool = False, rope_style: int = 0, inv_freq=None,
                  layer_inv_freq=None):
@@ -148,6 +152,8 @@ class CacheHitPath:
             off += nb
         host.copy_(dev.cpu())
         self._request_dev = dev
+        # served_pass's: one per layer's upload, one for the other joins
+        self._events = [torch.cuda.Event() for _ in range(L + 1)]
         self._layer_ranges = [(layer0 + l * layer_bytes, layer0 + (l + 1) * layer_bytes)
                               for l in range(L)]
         return host
@@ -176,38 +182,43 @@ class CacheHitPath:
         ``down_stream`` once its attention is done; the last layer's
         attention writes its rows into ``host_out`` itself (pinned host
         memory, reached over the chip-to-chip link).  Returns with the current stream
-        ordered after every copy.  Capturable in a CUDA graph."""
+        ordered after every copy; ``host`` and ``host_out`` have to stay alive
+        until it gets there.  Capturable in a CUDA graph."""
         L = self.wl.spec.layers
         main = torch.cuda.current_stream()
         dev = self._request_dev
-        fields_end = self._layer_ranges[0][0]
-        pic_copy_async(dev[:fields_end], host[:fields_end])
-        up_stream.wait_stream(main)
-        down_stream.wait_stream(main)
-        up_done = []
-        with torch.cuda.stream(up_stream):
-            for l in range(L):
-                lo, hi = self._layer_ranges[l]
-                if l == 0:
-                    pic_copy_async(dev[lo:hi], host[lo:hi])
-                else:
-                    dev[lo:hi].copy_(host[lo:hi], non_blocking=True)
-                up_done.append(torch.cuda.Event())
-                up_done[l].record(up_stream)
+        ev = self._events[L]
+
+        def after(waiter, on):  # work given to `waiter` from here on follows what `on` holds now
+            ev.record(on)
+            waiter.wait_event(ev)
+
+        self._copy(dev, host, 0, self._layer_ranges[0][0], False, main)
+        after(up_stream, main)
+        for l in range(L):
+            lo, hi = self._layer_ranges[l]
+            self._copy(dev, host, lo, hi - lo, l > 0, up_stream)
+            self._events[l].record(up_stream)
         for l in range(L):
             if l == 0:
                 self.link(-1)
-            main.wait_event(up_done[l])
+            main.wait_event(self._events[l])
             self.append(l)
             if l < L - 1:
                 self.attend(l)
-                down_stream.wait_stream(main)
-                with torch.cuda.stream(down_stream):
-                    host_out[l].copy_(self.out[l], non_blocking=True)
+                after(down_stream, main)
+                self._copy((host_out, l), (self.out, l), 0, -1, True, down_stream)
             else:
-                self.attend(l, out=host_out[l])  # the last layer's rows go straight to the host
-        main.wait_stream(up_stream)
-        main.wait_stream(down_stream)
+                self.attend(l, out=(host_out, l))  # the last layer's rows go straight to the host
+        after(main, up_stream)
+        if L > 1:
+            after(main, down_stream)
+
+    @staticmethod
+    def _copy(dst, src, offset, nbytes, engine, stream):
+        st = _native().copy_range(dst, src, offset, nbytes, engine, stream)
+        if st:
+            _check(st, "served_pass copy")
 
     # -- a1: layout and slot map
     def compose(self):
@@ -246,9 +257,9 @@ class CacheHitPath:
         pic_link(self.geom, wl.doc_len, wl.doc_base_pos, wl.doc_token_start, wl.req_doc_ids,
                  wl.req_num_docs, wl.prefix_len, wl.query_len, wl.block_table, wl.num_pages,
                  self.max_ctx, self.max_inline, wl.k_pool, wl.v_pool, 0, L, append_layer,
-                 wl.q_inline[append_layer] if app else None,
-                 wl.k_inline[append_layer] if app else None,
-                 wl.v_inline[append_layer] if app else None, wl.inline_len if app else None,
+                 (wl.q_inline, append_layer) if app else None,
+                 (wl.k_inline, append_layer) if app else None,
+                 (wl.v_inline, append_layer) if app else None, wl.inline_len if app else None,
                  self.k_cache, self.v_cache, self.doc_offset, self.doc_delta, self.slot_mapping,
                  self.tok_map, self.inline_pos, self.ctx_len, self.ws_prefill if app else None,
                  span_len=wl.span_len)
@@ -256,8 +267,8 @@ class CacheHitPath:
     # -- a4: RoPE + append of the inline tokens of one layer
     def append(self, layer: int):
         wl = self.wl
-        pic_append_inline(self.geom, layer, wl.q_inline[layer], wl.k_inline[layer],
-                          wl.v_inline[layer], self.inline_pos, wl.inline_len, self.slot_mapping,
+        pic_append_inline(self.geom, layer, (wl.q_inline, layer), (wl.k_inline, layer),
+                          (wl.v_inline, layer), self.inline_pos, wl.inline_len, self.slot_mapping,
                           wl.num_pages, self.k_cache, self.v_cache, self.ws_prefill)
 
     # -- a5: prefill attention of one layer
@@ -267,8 +278,8 @@ class CacheHitPath:
         wl = self.wl
         pic_attend_prefill(self.geom, layer, self.inline_pos, wl.inline_len, self.max_ctx,
                            wl.block_table, wl.num_pages, self.k_cache, self.v_cache,
-                           self.out[layer] if out is None else out,
-                           None if self.lse is None else self.lse[layer],
+                           (self.out, layer) if out is None else out,
+                           None if self.lse is None else (self.lse, layer),
                            self.prefill_splits, self.ws_prefill)
 
     # -- a7: prefill attention reading the documents from the pool (no relocate)
@@ -279,8 +290,8 @@ class CacheHitPath:
         pic_attend_prefill_fused(self.geom, layer, self.inline_pos, wl.inline_len, self.max_ctx,
                                  wl.block_table, wl.num_pages, self.k_cache, self.v_cache,
                                  wl.k_pool, wl.v_pool, self.tok_map, self.doc_delta,
-                                 self.out[layer] if out is None else out,
-                                 None if self.lse is None else self.lse[layer],
+                                 (self.out, layer) if out is None else out,
+                                 None if self.lse is None else (self.lse, layer),
                                  self.prefill_splits, self.ws_prefill)
 
     def prefill(self, layer: int):
@@ -290,9 +301,9 @@ class CacheHitPath:
         wl = self.wl
         pic_attend_prefill(self.geom, layer, self.inline_pos, wl.inline_len, self.max_ctx,
                            wl.block_table, wl.num_pages, self.k_cache, self.v_cache,
-                           self.out[layer], None if self.lse is None else self.lse[layer],
-                           self.prefill_splits, self.ws_prefill, q=wl.q_inline[layer],
-                           k_new=wl.k_inline[layer], v_new=wl.v_inline[layer])
+                           (self.out, layer), None if self.lse is None else (self.lse, layer),
+                           self.prefill_splits, self.ws_prefill, q=(wl.q_inline, layer),
+                           k_new=(wl.k_inline, layer), v_new=(wl.v_inline, layer))
 
     def fused_pass(self):
         """The cache-hit path with rotate-on-load attention: layout, then per
@@ -305,10 +316,10 @@ class CacheHitPath:
     # -- a6: one decode step of one layer (token position ctx_len + step)
     def decode(self, step: int, layer: int):
         wl = self.wl
-        pic_attend_decode(self.geom, layer, wl.q_dec[step, layer], wl.k_dec[step, layer],
-                          wl.v_dec[step, layer], self.ctx_len, wl.block_table, wl.num_pages,
-                          self.k_cache, self.v_cache, self.dec_out[layer], self.max_ctx,
-                          None if self.dec_lse is None else self.dec_lse[layer],
+        pic_attend_decode(self.geom, layer, (wl.q_dec, step, layer), (wl.k_dec, step, layer),
+                          (wl.v_dec, step, layer), self.ctx_len, wl.block_table, wl.num_pages,
+                          self.k_cache, self.v_cache, (self.dec_out, layer), self.max_ctx,
+                          None if self.dec_lse is None else (self.dec_lse, layer),
                           self.decode_splits, self.ws_decode, pos_offset=step)
 
     def ttft_pass(self, linked: bool = True):
