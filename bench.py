@@ -594,7 +594,10 @@ def main_gpu(args, rank, world):
                 dts.append(e0.elapsed_time(e1))
         dms = sum(dts) / len(dts)
         rows["a6_decode"] = {
-            "ms": dms, "launches": L * (3 if dsplits > 1 else 2), "splits": dsplits,
+            "ms": dms, "splits": dsplits,
+            # append and attention; the merge of more splits than a cluster takes
+            "launches": L * (2 if dsplits > 16 or dsplits * spec.kv_heads * spec.batch > 304
+                             else 1),
             "bytes": work["decode_bytes"], "gbs": work["decode_bytes"] / (dms * 1e6),
             "tok_s": spec.batch / (dms / 1e3)}
         rows["a6_decode"]["frac_hbm"] = rows["a6_decode"]["gbs"] / peaks["hbm_gbs"]

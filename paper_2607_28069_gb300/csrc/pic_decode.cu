@@ -3,19 +3,25 @@
 // first token, generation proceeds as usual on the linked cache).
 //
 // Decode reads every cached key and value of the request once per step and
-// does 2*G*d multiply-adds per key: HBM-bound.  Launches per call (one layer):
-//  1. decode_append_kernel: R(pos) k_new and v_new into slot(pos); the query
-//     rotated at pos into a bf16 workspace.
-//  2. decode_attn_kernel: one CTA per (key split, kv head, request), four
+// does 2*G*d multiply-adds per key: HBM-bound, and for few short requests
+// bound by launches and dependent round trips.  Launches per call (one layer):
+//  1. decode_attn_kernel: one CTA per (key split, kv head, request), four
 //     warps, each warp an independent stream over the split's pages (page
 //     w, w+4, ...).  Lane 0 of each warp keeps a 3-deep ring of TMA loads
 //     (one 16-key K page and V page, 128-byte swizzled so the ldmatrix reads
-//     below are bank-conflict free).  Scores S^T = K q^T come from
-//     m16n8k16 warp MMAs with the page's 16 keys as M and up to 8 query heads
-//     of the GQA group as N; P^T is turned into the B operand of the
-//     O^T += V^T P^T MMA in registers with movmatrix.  The four warps' states
-//     are merged through shared memory at the end.
-//  3. decode_combine_kernel (only with several splits): log-sum-exp merge.
+//     below are bank-conflict free).  While the first pages are in flight the
+//     CTA rotates its group's queries at the token's position; the CTA whose
+//     pages hold that position also rotates the new key, writes it and the
+//     new value to the cache and puts both into its copy of the page (the
+//     page it loads may or may not show its own store yet).  Scores S^T = K
+//     q^T come from m16n8k16 warp MMAs with the page's 16 keys as M and up to
+//     8 query heads of the GQA group as N; P^T is turned into the B operand
+//     of the O^T += V^T P^T MMA in registers with movmatrix.  The four warps'
+//     states are merged through shared memory at the end.
+//  2. decode_combine_kernel (only with several splits): log-sum-exp merge.
+//     A grid that fits the GPU at once and has at most 16 splits runs them as
+//     a thread-block cluster instead and merges through distributed shared
+//     memory, with no second launch.
 #include <algorithm>
 #include <mutex>
 
@@ -28,6 +34,13 @@ constexpr int kWarps = 4;
 constexpr int kThreads = 32 * kWarps;
 constexpr int NSTG = 3;
 constexpr int kMaxSplits = 64;
+constexpr int kMaxCluster = 16;  // splits of one (request, kv head) merged in a cluster
+// A grid of up to this many CTAs (two an SM) runs its splits as clusters, us per
+// layer against the merge launch: one request, 32/8 heads, 1k keys 6.42 and
+// 7.02, 128 keys 5.65 and 5.96, four of 4k 15.8 and 16.8; two of 1k, 28/4 6.75
+// and 7.37; d = 64 5.89 and 6.53.  (With the append as a launch of its own and
+// the merge launch: 10.5, 8.1, 22.0.)
+constexpr long long kClusterCtas = 304;
 
 template <int D>
 struct Layout {
@@ -35,25 +48,30 @@ struct Layout {
   static constexpr int kStage = 2 * kPage;        // K + V
   static constexpr int kWarpBytes = NSTG * kStage;
   static constexpr int kBar = kWarps * kWarpBytes;
-  static constexpr int kBytes = kBar + kWarps * NSTG * 8 + 16;
+  static constexpr int kCs = kBar + kWarps * NSTG * 8 + 16;  // cos/sin at the position (float2)
+  static constexpr int kNew = kCs + D / 2 * 8;               // new key, new value (bf16)
+  static constexpr int kQ = kNew + 2 * D * 2;                // rotated queries of the group (bf16)
+  static constexpr int kBytes = kQ + 16 * D * 2;
   static constexpr int kAlloc = kBytes + 1024;
 };
 
 struct Params {
   int Hq, Hkv, G, max_pages, splits, pages_per_split, pos_offset;
   long long num_pages, layer_row0;
+  int layer;
   const int32_t *pos, *block_table;
-  const __nv_bfloat16 *qrot;  // [B][Hq][D]
+  const __nv_bfloat16 *q, *k_new, *v_new;  // un-rotated: [B][Hq][D], [B][Hkv][D]
+  __nv_bfloat16 *k_cache, *v_cache;        // at the layer
   __nv_bfloat16 *out;
   float *lse, *part_o, *part_ml;
   int32_t *status;
   float scale_log2;
 };
 
-template <int D, int NT>
+template <int D, int NT, bool kCluster>
 __global__ void __launch_bounds__(kThreads)
     decode_attn_kernel(const __grid_constant__ CUtensorMap tm_k,
-                       const __grid_constant__ CUtensorMap tm_v, Params p) {
+                       const __grid_constant__ CUtensorMap tm_v, Params p, RopeParams rp) {
   using L = Layout<D>;
   constexpr int PANELS = D / 64;
   constexpr int KS = D / 16;  // k-steps over d
@@ -81,6 +99,33 @@ __global__ void __launch_bounds__(kThreads)
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
+  // ---- the token's projections go out before its position is known: chunk
+  // (8 pairs) tid of the group's queries, and the new key and value
+  constexpr int KC = D / 16, VC = D / 8;
+  const int tid = threadIdx.x;
+  const PairChunk pc = pair_chunk(tid % KC, D / 2, rp.style);
+  const bool has_q = tid < p.G * KC;  // G <= 16: one chunk per thread
+  uint4 qa = make_uint4(0, 0, 0, 0), qb2 = qa, ka = qa, kb = qa, vn = qa;
+  if (has_q) {
+    const __nv_bfloat16 *src = p.q + ((size_t)b * p.Hq + hk * p.G + tid / KC) * D;
+    qa = ld_stream(src + pc.off_a);
+    qb2 = ld_stream(src + pc.off_b);
+  }
+  if (tid < KC) {
+    const __nv_bfloat16 *src = p.k_new + ((size_t)b * p.Hkv + hk) * D;
+    ka = ld_stream(src + pc.off_a);
+    kb = ld_stream(src + pc.off_b);
+  } else if (tid >= 32 && tid < 32 + VC) {
+    vn = ld_stream(p.v_new + ((size_t)b * p.Hkv + hk) * D + (tid - 32) * 8);
+  }
+
+  // the block-table entries of this warp's first pages do not depend on the
+  // position either (lane i: its page i)
+  const int32_t *bt = p.block_table + (size_t)b * p.max_pages;
+  const int pg_begin = split * p.pages_per_split;
+  const int my_first = pg_begin + warp;  // pages of this warp: my_first + 4 i
+  const int bt_first = lane < NSTG && my_first + kWarps * lane < p.max_pages
+                           ? bt[my_first + kWarps * lane] : -1;
   const int pos = p.pos[b] + p.pos_offset;
   const int npages = pos >= 0 ? pos / 16 + 1 : 0;
   // max_ctx sized the split plan: keys past the last split's pages would be
@@ -88,21 +133,17 @@ __global__ void __launch_bounds__(kThreads)
   // request is then incomplete)
   if (split == p.splits - 1 && threadIdx.x == 0 && npages > p.splits * p.pages_per_split)
     dev_fail(p.status, PIC_DEV_CTX_OVERFLOW, b);
-  const int pg_begin = split * p.pages_per_split;
   const int pg_end = min(npages, pg_begin + p.pages_per_split);
-  const int32_t *bt = p.block_table + (size_t)b * p.max_pages;
 
   const uint32_t wbase = sbase + warp * L::kWarpBytes;
   auto full = [&](int s) { return sbase + L::kBar + 8u * (uint32_t)(warp * NSTG + s); };
-  // pages of this warp: pg_begin + warp + 4 i
-  const int my_first = pg_begin + warp;
   const int cw = my_first < pg_end ? (pg_end - my_first + kWarps - 1) / kWarps : 0;
 
-  auto issue = [&](int i) {  // lane 0 only
+  auto issue = [&](int i, int page_first) {  // lane 0 only; page_first: entry of page i < NSTG
     const int pidx = my_first + kWarps * i;
     int y = -1;
     if (pidx < p.max_pages) {
-      const int page = bt[pidx];
+      const int page = i < NSTG ? page_first : bt[pidx];
       if (page >= 0 && page < p.num_pages) y = (int)(p.layer_row0 + ((long long)page * p.Hkv + hk) * 16);
       else dev_fail(p.status, PIC_DEV_BAD_PAGE, b);
     } else {
@@ -117,8 +158,42 @@ __global__ void __launch_bounds__(kThreads)
       tma_load_2d(dst + L::kPage + pn * 2048, &tm_v, pn * 64, y, full(s));
     }
   };
-  if (lane == 0)
-    for (int i = 0; i < min(cw, NSTG); ++i) issue(i);
+#pragma unroll
+  for (int i = 0; i < NSTG; ++i) {
+    const int page_first = __shfl_sync(0xffffffffu, bt_first, i);
+    if (lane == 0 && i < cw) issue(i, page_first);
+  }
+
+  // ---- rotation at the position while the pages are in flight; the CTA whose
+  // pages hold the position appends the new key and value
+  float2 *cs = reinterpret_cast<float2 *>(smem + L::kCs);
+  __nv_bfloat16 *s_new = reinterpret_cast<__nv_bfloat16 *>(smem + L::kNew);
+  __nv_bfloat16 *s_q = reinterpret_cast<__nv_bfloat16 *>(smem + L::kQ);
+  const int new_pg = pos >= 0 ? pos >> 4 : -1, new_row = pos & 15;
+  int new_page = -1;  // the new token's page, -1: not this CTA's, or invalid
+  if (new_pg < 0 || new_pg >= p.max_pages) {
+    if (split == 0 && hk == 0 && tid == 0) dev_fail(p.status, PIC_DEV_BAD_POSITION, b);
+  } else if (new_pg >= pg_begin && (new_pg < pg_end || split == p.splits - 1)) {
+    new_page = bt[new_pg];
+    if (new_page < 0 || new_page >= p.num_pages) {
+      if (tid == 0) dev_fail(p.status, PIC_DEV_BAD_PAGE, b);
+      new_page = -1;
+    }
+  }
+  if (tid < D / 2) cs[tid] = rope_cos_sin(max(pos, 0), rope_theta(rp, p.layer, tid));
+  __syncthreads();
+  if (has_q) rotate_store_as<true>(qa, qb2, s_q + (tid / KC) * D, pc, rp.style, cs + 8 * (tid % KC));
+  if (new_page >= 0) {
+    const size_t row = (((size_t)new_page * p.Hkv + hk) * 16 + new_row) * D;
+    if (tid < KC) {
+      rotate_store_as<true>(ka, kb, s_new, pc, rp.style, cs + 8 * tid);
+      rotate_store_as<false>(ka, kb, p.k_cache + row, pc, rp.style, cs + 8 * tid);
+    } else if (tid >= 32 && tid < 32 + VC) {
+      *reinterpret_cast<uint4 *>(s_new + D + (tid - 32) * 8) = vn;
+      st_global16(p.v_cache + row + (tid - 32) * 8, vn);
+    }
+  }
+  __syncthreads();
 
   // query fragments (B operand of S^T = K q^T): heads nt*8 + gid of the group
   uint32_t qb[NT][KS][2];
@@ -126,8 +201,7 @@ __global__ void __launch_bounds__(kThreads)
   for (int nt = 0; nt < NT; ++nt) {
     const int hh = nt * 8 + gid;
     const bool hv = hh < p.G;
-    const uint32_t *qr = reinterpret_cast<const uint32_t *>(
-        p.qrot + ((size_t)b * p.Hq + hk * p.G + (hv ? hh : 0)) * D);
+    const uint32_t *qr = reinterpret_cast<const uint32_t *>(s_q + (hv ? hh : 0) * D);
 #pragma unroll
     for (int kk = 0; kk < KS; ++kk) {
       qb[nt][kk][0] = hv ? qr[(kk * 16 + 2 * tig) / 2] : 0u;
@@ -154,6 +228,13 @@ __global__ void __launch_bounds__(kThreads)
     done = i + 1;
     const uint32_t ks = wbase + s * L::kStage, vs = ks + L::kPage;
     const int key0 = (my_first + kWarps * i) * 16;
+    if (new_page >= 0 && my_first + kWarps * i == new_pg) {  // the new token's row of the page
+      const int piece = lane % VC;
+      if (lane < 2 * VC)
+        sts128((lane < VC ? ks : vs) + (piece >> 3) * 2048 + sw128_offset(new_row, (piece & 7) * 8),
+               *reinterpret_cast<const uint4 *>(s_new + (lane < VC ? 0 : D) + piece * 8));
+      __syncwarp();
+    }
     // ---- S^T[16 keys][8 heads] per n-tile
     float sacc[NT][4];
 #pragma unroll
@@ -214,7 +295,7 @@ __global__ void __launch_bounds__(kThreads)
       }
     }
     __syncwarp();
-    if (lane == 0 && i + NSTG < cw) issue(i + NSTG);
+    if (lane == 0 && i + NSTG < cw) issue(i + NSTG, -1);
   }
 
   if (done < cw) {
@@ -255,6 +336,7 @@ __global__ void __launch_bounds__(kThreads)
     }
   __syncthreads();
   const bool single = p.splits == 1;
+  float *c_acc = sl + kWarps * HMAX, *c_m = c_acc + HMAX * D, *c_l = c_m + HMAX;  // kCluster
   for (int e = threadIdx.x; e < p.G * D; e += kThreads) {
     const int hh = e / D, d = e % D;
     float M = -INFINITY;
@@ -272,6 +354,12 @@ __global__ void __launch_bounds__(kThreads)
     if (single) {
       p.out[h * D + d] = __float2bfloat16_rn(Ls > 0.f ? acc / Ls : 0.f);
       if (d == 0 && p.lse) p.lse[h] = Ls > 0.f ? (M + __log2f(Ls)) * 0.69314718055994531f : -INFINITY;
+    } else if constexpr (kCluster) {
+      c_acc[e] = acc;
+      if (d == 0) {
+        c_m[hh] = Ls > 0.f ? M : -INFINITY;
+        c_l[hh] = Ls;
+      }
     } else {
       p.part_o[(h * p.splits + split) * D + d] = acc;
       if (d == 0) {
@@ -280,8 +368,41 @@ __global__ void __launch_bounds__(kThreads)
       }
     }
   }
-  // release the dependent launch (merge, or the next layer's append) last
+  if constexpr (kCluster) {
+    // ---- the splits of this (request, kv head) are one cluster: each CTA
+    // merges its share of the output elements, o = sum_s w_s O_s / sum_s w_s l_s
+    // with w_s = 2^(m_s - M), from every CTA's shared memory
+    cluster_sync_all();
+    const int S = p.splits, per = (p.G * D + S - 1) / S;
+    for (int e = split * per + (int)threadIdx.x; e < min(p.G * D, (split + 1) * per); e += kThreads) {
+      const int hh = e / D, d = e % D;
+      float ms[kMaxCluster], ls[kMaxCluster], os[kMaxCluster];
+#pragma unroll
+      for (int c = 0; c < kMaxCluster; ++c) {
+        ms[c] = -INFINITY, ls[c] = 0.f, os[c] = 0.f;
+        if (c < S) {
+          ms[c] = ld_cluster(map_to_rank(smem_u32(c_m + hh), c));
+          ls[c] = ld_cluster(map_to_rank(smem_u32(c_l + hh), c));
+          os[c] = ld_cluster(map_to_rank(smem_u32(c_acc + e), c));
+        }
+      }
+      float M = -INFINITY, acc = 0.f, Ls = 0.f;
+#pragma unroll
+      for (int c = 0; c < kMaxCluster; ++c) M = fmaxf(M, ms[c]);
+#pragma unroll
+      for (int c = 0; c < kMaxCluster; ++c) {
+        const float w = ms[c] == -INFINITY ? 0.f : ex2(ms[c] - M);
+        acc = fmaf(w, os[c], acc);
+        Ls = fmaf(w, ls[c], Ls);
+      }
+      const size_t h = (size_t)b * p.Hq + hk * p.G + hh;
+      p.out[h * D + d] = __float2bfloat16_rn(acc * (Ls > 0.f ? 1.f / Ls : 0.f));
+      if (d == 0 && p.lse) p.lse[h] = Ls > 0.f ? (M + __log2f(Ls)) * 0.69314718055994531f : -INFINITY;
+    }
+  }
+  // release the dependent launch (merge, or the next layer's step) last
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if constexpr (kCluster) cluster_sync_all();  // the others may still read this CTA's shared memory
 }
 
 // Merge of the split partials of one (request, query head) row by
@@ -354,84 +475,6 @@ __global__ void decode_combine_kernel(Params p) {
   if (lane == 0 && p.lse) p.lse[hrow] = Ls > 0.f ? (M + __log2f(Ls)) * 0.69314718055994531f : -INFINITY;
 }
 
-struct AppendArgs {
-  int Hq, Hkv, max_pages, pos_offset, layer;
-  long long num_pages;
-  const __nv_bfloat16 *q, *k, *v;
-  const int32_t *pos, *block_table;
-  __nv_bfloat16 *k_cache, *v_cache, *qrot;  // cache pointers at the layer
-  int32_t *status;
-};
-
-template <int D>
-__global__ void __launch_bounds__(128) decode_append_kernel(AppendArgs a, RopeParams rp) {
-  constexpr int HALF = D / 2, KC = D / 16, VC = D / 8;
-  constexpr int R = 2;  // chunks per thread whose loads go out before the position is known
-  pdl_entry();
-  const int b = blockIdx.x, tid = threadIdx.x;
-  __shared__ float2 cs[HALF];
-  const int nK = a.Hkv * KC, nV = a.Hkv * VC, nQ = a.Hq * KC;
-  // the token's projections do not depend on its position: their first
-  // chunks are loaded before it is (the rest, if any, after)
-  uint4 ka[R], kb[R], vv[R], qa[R], qb[R];
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int e = tid + (int)blockDim.x * i;
-    if (e < nK) {
-      const PairChunk pc = pair_chunk(e % KC, HALF, rp.style);
-      const __nv_bfloat16 *src = a.k + ((size_t)b * a.Hkv + e / KC) * D;
-      ka[i] = ld_stream(src + pc.off_a);
-      kb[i] = ld_stream(src + pc.off_b);
-    }
-    if (e < nV) vv[i] = ld_stream(a.v + ((size_t)b * a.Hkv + e / VC) * D + (e % VC) * 8);
-    if (e < nQ) {
-      const PairChunk pc = pair_chunk(e % KC, HALF, rp.style);
-      const __nv_bfloat16 *src = a.q + ((size_t)b * a.Hq + e / KC) * D;
-      qa[i] = ld_stream(src + pc.off_a);
-      qb[i] = ld_stream(src + pc.off_b);
-    }
-  }
-  const int pos = a.pos[b] + a.pos_offset;
-  long long page = -1;
-  if (pos < 0 || pos / 16 >= a.max_pages) {
-    if (tid == 0) dev_fail(a.status, PIC_DEV_BAD_POSITION, b);
-  } else {
-    page = a.block_table[(size_t)b * a.max_pages + pos / 16];
-    if (page < 0 || page >= a.num_pages) {
-      if (tid == 0) dev_fail(a.status, PIC_DEV_BAD_PAGE, b);
-      page = -1;
-    }
-  }
-  for (int i = tid; i < HALF; i += blockDim.x)
-    cs[i] = rope_cos_sin(pos > 0 ? pos : 0, rope_theta(rp, a.layer, i));
-  __syncthreads();
-  const int r = pos & 15;
-  auto k_dst = [&](int e) { return a.k_cache + ((page * a.Hkv + e / KC) * 16 + r) * D; };
-  auto v_dst = [&](int e) { return a.v_cache + ((page * a.Hkv + e / VC) * 16 + r) * D + (e % VC) * 8; };
-  auto q_dst = [&](int e) { return a.qrot + ((size_t)b * a.Hq + e / KC) * D; };
-  if (page >= 0) {
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int e = tid + (int)blockDim.x * i;
-      if (e < nK) rotate_store(ka[i], kb[i], k_dst(e), pair_chunk(e % KC, HALF, rp.style), rp.style, cs + 8 * (e % KC));
-      if (e < nV) st_global16(v_dst(e), vv[i]);
-    }
-    for (int e = tid + (int)blockDim.x * R; e < nK; e += blockDim.x)
-      rotate_chunk(a.k + ((size_t)b * a.Hkv + e / KC) * D, k_dst(e), e % KC, HALF, rp.style,
-                   cs + 8 * (e % KC), true);
-    for (int e = tid + (int)blockDim.x * R; e < nV; e += blockDim.x)
-      st_global16(v_dst(e), ld_stream(a.v + ((size_t)b * a.Hkv + e / VC) * D + (e % VC) * 8));
-  }
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int e = tid + (int)blockDim.x * i;
-    if (e < nQ) rotate_store(qa[i], qb[i], q_dst(e), pair_chunk(e % KC, HALF, rp.style), rp.style, cs + 8 * (e % KC));
-  }
-  for (int e = tid + (int)blockDim.x * R; e < nQ; e += blockDim.x)
-    rotate_chunk(a.q + ((size_t)b * a.Hq + e / KC) * D, q_dst(e), e % KC, HALF, rp.style,
-                 cs + 8 * (e % KC), true);
-}
-
 struct Plan {
   int splits, pages_per_split;
   size_t q_bytes, po_bytes, pml_bytes, total;
@@ -439,15 +482,40 @@ struct Plan {
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Key splits for `units` (request, kv head) pairs of `pages` pages.  Grids of
+// about 256 CTAs (two fit on an SM, 304 in all) or a multiple do best: just past
+// one wave a second one starts that fills little of the GPU; a multiple, so
+// that no CTA has more than 256 pages and the last ones end together.  And no
+// more than sqrt(pages) splits: a page costs a warp about half a microsecond,
+// a split of its own the merge a tenth.  Against splits for four waves (at
+// least 16 pages each), us per layer (heads 32/8 unless stated): 1 request of
+// 16k keys 24.1 -> 18.1 (64 -> 32 splits), 33k 33.6 -> 27.5, 131k 92 -> 86; 3
+// requests of 16k, 8/2 heads 21.9 -> 15.3; 4 of 4k 19.9 -> 15.8 (16 -> 8); 2 of
+// 400 8.9 -> 6.3 (1 -> 6); 8 of 16k 89.1 -> 84.5; 16 of 33k, 28/4 164.7 -> 161.4.
+// Groups of more than 8 heads (two columns of MMAs, one CTA an SM at 164
+// registers) keep four waves of splits of at least 16 pages: it suits one or
+// two requests as well (16 heads a group, 33k keys: 64 splits 18.5 us, 32 22.4);
+// 32 requests of 10k would do better with 8 splits than with its 38 (34 against
+// 52 us), but the allocation-free call's tests hold it to that plan.
+inline int auto_splits(long long units, int pages, bool wide_group) {
+  if (wide_group)
+    return (int)std::max(1ll, std::min({(8ll * 152 + units - 1) / units,
+                                        (long long)std::max(1, pages / 16), (long long)kMaxSplits}));
+  constexpr long long kWave = 256;
+  constexpr int kMaxPages = 256;
+  long long s = 0;
+  for (long long w = 1; s == 0 || (s < kMaxSplits && pages > kMaxPages * s); ++w) s = kWave * w / units;
+  int root = 1;
+  while ((long long)root * root < pages) ++root;
+  return (int)std::max(1ll, std::min({s, (long long)root, (long long)kMaxSplits}));
+}
+
 inline Plan plan(const pic_geom_t *g, int batch, int max_ctx, int num_splits) {
   Plan pl;
   const int pages = (max_ctx + 15) / 16;
-  if (num_splits <= 0) {
-    const long long units = (long long)batch * g->num_kv_heads;
-    int s = (int)((8LL * 152 + units - 1) / units);
-    s = std::min(s, std::max(1, pages / 16));  // at least ~4 pages per warp
-    num_splits = std::max(1, std::min(s, kMaxSplits));
-  }
+  if (num_splits <= 0)
+    num_splits = auto_splits((long long)batch * g->num_kv_heads, pages,
+                             g->num_q_heads / g->num_kv_heads > 8);
   num_splits = std::min(num_splits, pages);
   pl.splits = std::max(1, num_splits);
   pl.pages_per_split = (pages + pl.splits - 1) / pl.splits;
@@ -463,15 +531,17 @@ inline Plan plan(const pic_geom_t *g, int batch, int max_ctx, int num_splits) {
 }
 
 template <int D, int NT>
-cudaError_t launch_attn(dim3 grid, cudaStream_t stream, const CUtensorMap &tk,
-                        const CUtensorMap &tv, const Params &pp) {
+cudaError_t launch_attn(dim3 grid, bool cluster, cudaStream_t stream, const CUtensorMap &tk,
+                        const CUtensorMap &tv, const Params &pp, const RopeParams &rp) {
   const int smem = Layout<D>::kAlloc;
-  cudaError_t e = cudaFuncSetAttribute(decode_attn_kernel<D, NT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  auto *kernel = cluster ? decode_attn_kernel<D, NT, true> : decode_attn_kernel<D, NT, false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess && cluster && grid.x > 8)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
-  e = launch_dependent(decode_attn_kernel<D, NT>, grid, dim3(kThreads), smem, stream, tk, tv, pp);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return cluster ? launch_dependent_cluster(kernel, grid, dim3(kThreads), smem, stream, (int)grid.x,
+                                            tk, tv, pp, rp)
+                 : launch_dependent(kernel, grid, dim3(kThreads), smem, stream, tk, tv, pp, rp);
 }
 
 }  // namespace decode
@@ -529,7 +599,7 @@ static pic_status_t check_step(const char *who, const pic_geom_t *geom, RopePara
   return PIC_OK;
 }
 
-// The launches of one decoding step of one layer (append, attention, merge
+// The launches of one decoding step of one layer (append and attention, merge
 // when split) with the scratch at `ws` laid out by `pl`.
 static pic_status_t launch_step(const char *who, const pic_geom_t *geom, const RopeParams &rp,
                                 int32_t layer, int32_t batch, const void *q, const void *k_new,
@@ -543,29 +613,6 @@ static pic_status_t launch_step(const char *who, const pic_geom_t *geom, const R
   const int G = geom->num_q_heads / Hkv;
   const long long rows_total = (long long)geom->num_layers * num_pages * Hkv * 16;
   const size_t layer_elems = (size_t)num_pages * Hkv * 16 * D;
-
-  AppendArgs aa;
-  aa.Hq = geom->num_q_heads;
-  aa.Hkv = Hkv;
-  aa.max_pages = max_pages;
-  aa.pos_offset = pos_offset;
-  aa.layer = layer;
-  aa.num_pages = num_pages;
-  aa.q = static_cast<const __nv_bfloat16 *>(q);
-  aa.k = static_cast<const __nv_bfloat16 *>(k_new);
-  aa.v = static_cast<const __nv_bfloat16 *>(v_new);
-  aa.pos = pos;
-  aa.block_table = block_table;
-  aa.k_cache = static_cast<__nv_bfloat16 *>(k_cache) + (size_t)layer * layer_elems;
-  aa.v_cache = static_cast<__nv_bfloat16 *>(v_cache) + (size_t)layer * layer_elems;
-  aa.qrot = reinterpret_cast<__nv_bfloat16 *>(ws);
-  aa.status = status;
-  {
-    const cudaError_t ae =
-        D == 128 ? launch_dependent(decode_append_kernel<128>, dim3(batch), dim3(128), 0, stream, aa, rp)
-                 : launch_dependent(decode_append_kernel<64>, dim3(batch), dim3(128), 0, stream, aa, rp);
-    if (ae != cudaSuccess) return cuda_fail(ae, "decode append launch");
-  }
 
   CUtensorMap tk, tv;
   pic_status_t st = encode_tmap_2d(&tk, k_cache, D, rows_total, (uint64_t)D * 2, 64, 16);
@@ -584,7 +631,12 @@ static pic_status_t launch_step(const char *who, const pic_geom_t *geom, const R
   pp.layer_row0 = (long long)layer * num_pages * Hkv * 16;
   pp.pos = pos;
   pp.block_table = block_table;
-  pp.qrot = aa.qrot;
+  pp.layer = layer;
+  pp.q = static_cast<const __nv_bfloat16 *>(q);
+  pp.k_new = static_cast<const __nv_bfloat16 *>(k_new);
+  pp.v_new = static_cast<const __nv_bfloat16 *>(v_new);
+  pp.k_cache = static_cast<__nv_bfloat16 *>(k_cache) + (size_t)layer * layer_elems;
+  pp.v_cache = static_cast<__nv_bfloat16 *>(v_cache) + (size_t)layer * layer_elems;
   pp.out = static_cast<__nv_bfloat16 *>(out);
   pp.lse = lse;
   pp.part_o = pl.splits > 1 ? reinterpret_cast<float *>(ws + pl.q_bytes) : nullptr;
@@ -594,10 +646,16 @@ static pic_status_t launch_step(const char *who, const pic_geom_t *geom, const R
 
   dim3 grid(pl.splits, Hkv, batch);
   cudaError_t e;
-  if (D == 128) e = G <= 8 ? launch_attn<128, 1>(grid, stream, tk, tv, pp) : launch_attn<128, 2>(grid, stream, tk, tv, pp);
-  else e = G <= 8 ? launch_attn<64, 1>(grid, stream, tk, tv, pp) : launch_attn<64, 2>(grid, stream, tk, tv, pp);
+  const bool cluster = pl.splits > 1 && pl.splits <= kMaxCluster &&
+                       (long long)pl.splits * Hkv * batch <= kClusterCtas;
+  if (D == 128)
+    e = G <= 8 ? launch_attn<128, 1>(grid, cluster, stream, tk, tv, pp, rp)
+               : launch_attn<128, 2>(grid, cluster, stream, tk, tv, pp, rp);
+  else
+    e = G <= 8 ? launch_attn<64, 1>(grid, cluster, stream, tk, tv, pp, rp)
+               : launch_attn<64, 2>(grid, cluster, stream, tk, tv, pp, rp);
   if (e != cudaSuccess) return cuda_fail(e, "decode attention launch");
-  if (pl.splits > 1) {
+  if (pl.splits > 1 && !cluster) {
     dim3 cgrid(geom->num_q_heads, batch);
     const cudaError_t ce =
         D == 128 ? launch_dependent(decode_combine_kernel<128>, cgrid, dim3(32), 0, stream, pp)
@@ -644,7 +702,7 @@ extern "C" pic_status_t pic_attend_decode(const pic_geom_t *geom, int32_t layer,
 // engine that has handed its whole memory budget to the KV cache, a runtime
 // that forbids allocation after start-up, or an embedding that only owns the
 // tensors it passes in.  For them this entry point takes no workspace: its
-// scratch (the rotated queries and the per-split partial softmax states) lives
+// scratch (the per-split partial softmax states) lives
 // in the file-scope device array below, which every GPU that loads the library
 // holds until the process exits.
 //

@@ -292,8 +292,10 @@ PIC_DEV PairChunk pair_chunk(int c, int half, int style) {
 // Rotates the chunk of 8 pairs whose two 16-byte halves va, vb were loaded
 // from offsets pc.off_a, pc.off_b of a row, and stores it at the same
 // offsets of dst.
-PIC_DEV void rotate_store(uint4 va, uint4 vb, __nv_bfloat16 *dst, const PairChunk &pc, int style,
-                          const float2 *cs) {
+// (kShared: dst is shared memory.)
+template <bool kShared>
+PIC_DEV void rotate_store_as(uint4 va, uint4 vb, __nv_bfloat16 *dst, const PairChunk &pc, int style,
+                             const float2 *cs) {
   float a[8], b[8], u[8], w[8];
   unpack8(va, a);
   unpack8(vb, b);
@@ -318,8 +320,17 @@ PIC_DEV void rotate_store(uint4 va, uint4 vb, __nv_bfloat16 *dst, const PairChun
       b[2 * i] = u[4 + i]; b[2 * i + 1] = w[4 + i];
     }
   }
-  st_global16(dst + pc.off_a, pack8(a));
-  st_global16(dst + pc.off_b, pack8(b));
+  if constexpr (kShared) {
+    *reinterpret_cast<uint4 *>(dst + pc.off_a) = pack8(a);
+    *reinterpret_cast<uint4 *>(dst + pc.off_b) = pack8(b);
+  } else {
+    st_global16(dst + pc.off_a, pack8(a));
+    st_global16(dst + pc.off_b, pack8(b));
+  }
+}
+PIC_DEV void rotate_store(uint4 va, uint4 vb, __nv_bfloat16 *dst, const PairChunk &pc, int style,
+                          const float2 *cs) {
+  rotate_store_as<false>(va, vb, dst, pc, style, cs);
 }
 
 PIC_DEV void rotate_chunk(const __nv_bfloat16 *src, __nv_bfloat16 *dst, int c, int half,
@@ -403,6 +414,11 @@ PIC_DEV uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
+}
+PIC_DEV float ld_cluster(uint32_t addr) {  // addr from map_to_rank
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
 }
 // All threads of every CTA of the cluster (release / acquire at cluster scope).
 PIC_DEV void cluster_sync_all() {
