@@ -1466,8 +1466,12 @@ extern "C" int32_t pic_prefill_num_splits(const pic_geom_t *geom, int32_t batch,
 // pair, key split, kv head and request, a pair's tiles counted from the
 // request's last packed row as the kernel does) are dealt greedily to the
 // SMs, each costing its key tiles plus a fixed per-CTA cost, and the count
-// with the least makespan (plus a merge cost when split) wins; a grid that
-// fits in one wave with the library's count is not split further.
+// with the least makespan plus merge cost wins.  The constants fit sweeps of the
+// count (us of attention and merge, one layer, 32/8 heads): 8 requests of 16.8k
+// keys, 256 query tokens: 360 with 1 split, 392 / 406 / 390 with 2 / 3 / 4 (4
+// before); with spans 899 and 999 / 1018 / 1037 (3 before), rotate-on-load 1174
+// and 1300; 2 requests of 4k 28.1 with 4, 28.9 with 3; 4 of 8k, 16/2 heads of
+// 64, 30.7 with 4, 34.6 with 3; 4 of 139k 2886 with 1, 2832-2874 with 4 to 10.
 extern "C" int32_t pic_prefill_plan_splits(const pic_geom_t *geom, int32_t batch,
                                            int32_t max_inline, int32_t max_ctx,
                                            const int32_t *inline_len, const int32_t *inline_pos) {
@@ -1491,16 +1495,27 @@ extern "C" int32_t pic_prefill_plan_splits(const pic_geom_t *geom, int32_t batch
       }
     }
   }
-  constexpr double kCtaFixed = 2.0, kCtaEmpty = 0.3, kMerge = 1.0;  // in key-tile times
+  // in key-tile times (1.3 us at d = 128): a CTA's set-up, fill and drain, an
+  // empty CTA, the merge launch and the 4 d + 16 bytes written and read per
+  // partial row at 6.5 TB/s
+  constexpr double kCtaFixed = 4.0, kCtaEmpty = 0.7, kMerge = 2.0, kTileBytes = 8.5e6;
+  const double kRowBytes = 4.0 * geom->head_dim + 16.0;
   constexpr int kSms = 152;
   double best = 1e300;
   int best_s = fallback;
   std::vector<double> sm(kSms);
-  // A grid the library's count already fits in one wave is latency-bound:
-  // more splits there only add merge traffic the estimate leaves out.
-  int max_s = std::min(kMaxSplits, std::max(1, kv_tiles));
-  if ((long long)batch * Hkv * npairs * fallback <= kSms) max_s = std::min(max_s, fallback);
+  const int max_s = std::min(kMaxSplits, std::max(1, kv_tiles));
   for (int sp = 1; sp <= max_s; ++sp) {
+    const double merge = kMerge + (double)batch * Hkv * m_tiles * BM * sp * kRowBytes / kTileBytes;
+    // no larger count can win once even a perfect balance costs more than the
+    // best: key tiles and fixed costs (of the splits that have keys) over the SMs
+    double work = 0.0;
+    for (int na : pair_tiles)
+      if (na > 0) {
+        const int per = (na + sp - 1) / sp;
+        work += na + kCtaFixed * ((na + per - 1) / per);
+      }
+    if (sp > 1 && work * Hkv / kSms + merge > best) break;
     std::fill(sm.begin(), sm.end(), 0.0);
     std::make_heap(sm.begin(), sm.end(), std::greater<double>());
     for (int b = 0; b < batch; ++b)
@@ -1514,7 +1529,7 @@ extern "C" int32_t pic_prefill_plan_splits(const pic_geom_t *geom, int32_t batch
           sm.back() += n > 0 ? n + kCtaFixed : kCtaEmpty;
           std::push_heap(sm.begin(), sm.end(), std::greater<double>());
         }
-    const double cost = *std::max_element(sm.begin(), sm.end()) + (sp > 1 ? kMerge : 0.0);
+    const double cost = *std::max_element(sm.begin(), sm.end()) + (sp > 1 ? merge : 0.0);
     if (cost < best - 1e-9) {
       best = cost;
       best_s = sp;
