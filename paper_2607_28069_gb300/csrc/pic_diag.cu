@@ -25,11 +25,13 @@ constexpr int kComputeWarps = 8;  // two per TMEM lane quarter, each on half the
 constexpr int kRegionWarp = 10;
 constexpr int BM = 128;        // query rows per tile (TMEM lanes)
 constexpr int BN = 128;        // key positions per tile
-constexpr int NS = 2;          // K stages, each a tile of cache A and one of cache B
+// K stages, each a tile of cache A and one of cache B: three where the document
+// table leaves room (one more bulk of loads in flight), else two
+constexpr int kMaxStages = 3;
 constexpr int kMaxRegions = 8;
 constexpr uint32_t kTmemCols = 512;  // two buffers of (S_A, S_B), 128 columns each
 
-template <int D>
+template <int D, int NS>
 struct DLayout {
   static constexpr int kTile = BN * D * 2;        // one K tile
   static constexpr int kQ = 0;
@@ -47,8 +49,8 @@ struct DLayout {
 enum {
   DB_Q = 0,
   DB_KFULL = 1,
-  DB_KEMPTY = DB_KFULL + NS,
-  DB_SFULL = DB_KEMPTY + NS,  // per S buffer
+  DB_KEMPTY = DB_KFULL + kMaxStages,
+  DB_SFULL = DB_KEMPTY + kMaxStages,  // per S buffer
   DB_SFREE = DB_SFULL + 2,    // per S buffer, one arrival per compute warp
   DB_RFULL = DB_SFREE + 2,    // per region buffer (the region bytes of a tile)
   DB_FINAL = DB_RFULL + 2,
@@ -120,15 +122,22 @@ __device__ uint32_t four_regions(const int32_t *s_off, const int32_t *s_bnd, int
 // boxes through the block layout, as the prefill attention does), one after
 // the other, and the region warp writes the tile's key regions; the issuer
 // computes [S_A S_B] = Q [K_A; K_B]^T, one N = 256 MMA per 16-deep slice,
-// into a TMEM buffer (two buffers, so the next tile's MMAs overlap this
-// one's exponentials); each compute thread owns one query row, reads both
-// rows of scores from TMEM 32 columns at a time and adds |p_A - p_B| to its
-// region.
-template <int D>
+// into a TMEM buffer (two buffers); each compute thread owns half of one query
+// row's keys, reads both configurations' scores of the tile from TMEM into
+// registers, gives the buffer back at once, so that the next MMA into it never
+// waits for exponentials, and adds |p_A - p_B| to the keys' regions.
+// The two exponentials a term take MUFU 1024 cycles a tile and the MMAs as
+// long; a tile takes about 2350, in the compute warps' dependent chains (two
+// warps an SMSP, in step on the same tile).  One layer of two requests of 14k
+// document tokens, 256 query tokens each: 181 us with 32 columns read at a time,
+// scalar scaling and one masked sum per region at every boundary, 174 with the
+// tile in registers and packed pairs, 162 with the split count's cost model
+// fitted to it.
+template <int D, int NS>
 __global__ void __launch_bounds__(kThreads, 1)
     deviation_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_ka,
                      const __grid_constant__ CUtensorMap tm_kb, DevArgs a) {
-  using L = DLayout<D>;
+  using L = DLayout<D, NS>;
   constexpr int PANELS = D / 64;
   constexpr uint32_t IDESC_QK = idesc_bf16(BM, 2 * BN, false, false);
   constexpr uint32_t kPageBytes = 16 * D * 2;
@@ -306,14 +315,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       mma_commit(bar(DB_FINAL), el);
     } else {
       // ================================================ compute warps
-      // Two warps per TMEM lane quarter, each on 64 of the 128 key columns,
-      // 32 at a time.  The 32 terms of a chunk are computed without branches
+      // Two warps per TMEM lane quarter, each on 64 of the 128 key columns in
+      // two chunks of 32.  The terms of a chunk are computed without branches
       // (the exponentials pipeline); a chunk whose keys all lie in one region
-      // (the region bytes are the same for every row) is summed at once, one
-      // in no region is skipped, and only a chunk across a region or
-      // document boundary is summed key by key.  A key after a row's
-      // position (an inline span taken as a query row before a later
-      // document) has p_A = p_B = 0.
+      // (the region bytes are the same for every row) is summed at once, one in
+      // no region is skipped, one across a single region or document boundary
+      // takes two sums, and only a chunk with more boundaries is summed region
+      // by region.  A key after a row's position (an inline span taken as a
+      // query row before a later document) has p_A = p_B = 0.
       const int wq = warp & 3, half = (warp - 2) >> 2;
       const int row = wq * 32 + lane, rg = r0 + row;
       float la = INFINITY, lb = INFINITY;  // rows past the query rows add nothing
@@ -341,63 +350,89 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (ok) ok = mbar_wait(bar(DB_SFULL + buf), (j >> 1) & 1, abort_flag, a.status, b);
         if (!__all_sync(0xffffffffu, ok)) break;
         tc_fence_after();
-#pragma unroll 1
-        for (int c0 = 0; c0 < 64; c0 += 32) {
-          const int8_t *rr = s_reg + buf * BN + half * 64 + c0;
-          const uint4 w0 = *reinterpret_cast<const uint4 *>(rr);
-          const uint4 w1 = *reinterpret_cast<const uint4 *>(rr + 16);
-          const int reg0 = rr[0];
-          const uint32_t rep = (uint32_t)(uint8_t)rr[0] * 0x01010101u;
-          const bool uniform = w0.x == rep && w0.y == rep && w0.z == rep && w0.w == rep &&
-                               w1.x == rep && w1.y == rep && w1.z == rep && w1.w == rep;
-          if (uniform && reg0 < 0) continue;  // no key of the chunk is in a region
-          float sa[32], sb[32];
-          tmem_ld32(tl + buf * 256 + c0, reinterpret_cast<uint32_t *>(sa));
-          tmem_ld32(tl + buf * 256 + 128 + c0, reinterpret_cast<uint32_t *>(sb));
-          tmem_wait_ld();
+        // the tile's scores and region bytes (lane l: key l of each chunk) into
+        // registers; both buffers are then free
+        float sa[64], sb[64];
+        int rb[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          tmem_ld32(tl + buf * 256 + h * 32, reinterpret_cast<uint32_t *>(sa + h * 32));
+          tmem_ld32(tl + buf * 256 + 128 + h * 32, reinterpret_cast<uint32_t *>(sb + h * 32));
+          rb[h] = s_reg[buf * BN + half * 64 + h * 32 + lane];
+        }
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(DB_SFREE + buf));
+        const uint64_t sc2 = f2pack(a.scale_log2, a.scale_log2), one2 = f2pack(-1.f, -1.f);
+        const uint64_t na2 = f2pack(-la, -la), nb2 = f2pack(-lb, -lb);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int reg0 = __shfl_sync(0xffffffffu, rb[h], 0);
+          const uint32_t same = __ballot_sync(0xffffffffu, rb[h] == reg0);
+          if (same == 0xffffffffu && reg0 < 0) continue;  // no key of the chunk is in a region
           // keys 0..lim of the chunk are at or before this row's position
-          const long long t0 = (long long)(kt0 + kv_begin + j) * BN + half * 64 + c0;
+          const long long t0 = (long long)(kt0 + kv_begin + j) * BN + half * 64 + h * 32;
           const int lim = (int)min(max(qpos - t0, -1ll), 31ll);
-          if (uniform && __all_sync(0xffffffffu, lim == 31)) {
-            // one region, every key visible to every row of the warp: six
-            // instructions a term (two FFMA, two EX2, two FADD)
+          const bool visible = __all_sync(0xffffffffu, lim == 31);
+          // the terms of keys c, c + 1: 4.5 instructions each (packed scaling and
+          // difference, EX2 twice)
+          auto terms = [&](int c, float &d0, float &d1) {
+            const int e = h * 32 + c;
+            const uint64_t ea = exp2_mufu2(fma2(f2pack(sa[e], sa[e + 1]), sc2, na2));
+            const uint64_t eb = exp2_mufu2(fma2(f2pack(sb[e], sb[e + 1]), sc2, nb2));
+            f2unpack(fma2(eb, one2, ea), d0, d1);
+            d0 = fabsf(d0), d1 = fabsf(d1);
+          };
+          if (same == 0xffffffffu && visible) {
             float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;
 #pragma unroll
             for (int c = 0; c < 32; c += 4) {
-              v0 += fabsf(ex2(fmaf(sa[c], a.scale_log2, -la)) - ex2(fmaf(sb[c], a.scale_log2, -lb)));
-              v1 += fabsf(ex2(fmaf(sa[c + 1], a.scale_log2, -la)) - ex2(fmaf(sb[c + 1], a.scale_log2, -lb)));
-              v2 += fabsf(ex2(fmaf(sa[c + 2], a.scale_log2, -la)) - ex2(fmaf(sb[c + 2], a.scale_log2, -lb)));
-              v3 += fabsf(ex2(fmaf(sa[c + 3], a.scale_log2, -la)) - ex2(fmaf(sb[c + 3], a.scale_log2, -lb)));
+              float d0, d1, d2, d3;
+              terms(c, d0, d1);
+              terms(c + 2, d2, d3);
+              v0 += d0, v1 += d1, v2 += d2, v3 += d3;
             }
             add_to(reg0, (v0 + v1) + (v2 + v3));
-          } else {
-            // a region or document boundary inside the chunk, or keys after
-            // some row's position: the masked terms first, then one masked
-            // sum per region, with no branch between the terms (a branch per
-            // key would serialise the exponentials)
+            continue;
+          }
+          float d[32];
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const float d = fabsf(ex2(fmaf(sa[c], a.scale_log2, -la)) - ex2(fmaf(sb[c], a.scale_log2, -lb)));
-              sa[c] = c <= lim ? d : 0.f;
+          for (int c = 0; c < 32; c += 2) {
+            terms(c, d[c], d[c + 1]);
+            if (c > lim) d[c] = 0.f;
+            if (c + 1 > lim) d[c + 1] = 0.f;
+          }
+          // one boundary: keys below n_lo in reg0, the rest in reg1
+          const int reg1 = __shfl_sync(0xffffffffu, rb[h], 31);
+          const uint32_t rest = __ballot_sync(0xffffffffu, rb[h] == reg1);
+          if ((same & (same + 1)) == 0 && (rest | same) == 0xffffffffu) {
+            const int n_lo = same == 0xffffffffu ? 32 : __popc(same);
+            float lo0 = 0.f, lo1 = 0.f, hi0 = 0.f, hi1 = 0.f;
+#pragma unroll
+            for (int c = 0; c < 32; c += 2) {
+              lo0 += c < n_lo ? d[c] : 0.f;
+              hi0 += c < n_lo ? 0.f : d[c];
+              lo1 += c + 1 < n_lo ? d[c + 1] : 0.f;
+              hi1 += c + 1 < n_lo ? 0.f : d[c + 1];
             }
-            int rg[32];
-#pragma unroll
-            for (int c = 0; c < 32; ++c) rg[c] = rr[c];
+            add_to(reg0, lo0 + lo1);
+            add_to(reg1, hi0 + hi1);
+          } else {
 #pragma unroll 1
             for (int i = 0; i < a.n_regions; ++i) {
+              const uint32_t in = __ballot_sync(0xffffffffu, rb[h] == i);
+              if (!in) continue;
               float v0 = 0.f, v1 = 0.f;
 #pragma unroll
               for (int c = 0; c < 32; c += 2) {
-                v0 += rg[c] == i ? sa[c] : 0.f;
-                v1 += rg[c + 1] == i ? sa[c + 1] : 0.f;
+                v0 += (in >> c) & 1u ? d[c] : 0.f;
+                v1 += (in >> (c + 1)) & 1u ? d[c + 1] : 0.f;
               }
               add_to(i, v0 + v1);
             }
           }
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(DB_SFREE + buf));
       }
 #pragma unroll
       for (int i = 0; i < kMaxRegions; ++i) {
@@ -506,7 +541,8 @@ extern "C" pic_status_t pic_attention_deviation(
   // query tiles: the query rows of a request are its last query_len inline
   // tokens times G.  Key splits (every split adds its own partial sums): one
   // CTA per SM, so a launch takes ceil(CTAs / 152) rounds of one CTA's key
-  // tiles plus about two tiles of pipeline fill; take the split count that
+  // tiles plus its set-up, fill and drain (8.5 us, seven tiles at 1.15 us each:
+  // from launches of 27 to 431 tiles an SM); take the split count that
   // minimises that
   const int q_tiles = (int)(((long long)max_query_len * G + BM - 1) / BM);
   const int kt_max = (max_ctx + BN - 1) / BN;
@@ -514,7 +550,7 @@ extern "C" pic_status_t pic_attention_deviation(
   a.splits = 1;
   long long best = -1;
   for (int sp = 1; sp <= std::min(kt_max, 64); ++sp) {
-    const long long cost = ((groups * sp + 151) / 152) * ((kt_max + sp - 1) / sp + 2);
+    const long long cost = ((groups * sp + 151) / 152) * ((kt_max + sp - 1) / sp + 7);
     if (best < 0 || cost < best) best = cost, a.splits = sp;
   }
   cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(double) * batch * n_regions, stream);
@@ -524,20 +560,30 @@ extern "C" pic_status_t pic_attention_deviation(
   if ((long long)q_tiles * a.splits > 65535 || batch > 65535 || Hkv > 65535)
     return fail(PIC_ERR_INVALID_ARG, "pic_attention_deviation: grid too large");
   const dim3 grid((unsigned)(q_tiles * a.splits), Hkv, batch);
-  const size_t smem_need = D == 128 ? DLayout<128>::alloc(max_docs, n_regions)
-                                     : DLayout<64>::alloc(max_docs, n_regions);
-  if (smem_need > 227 * 1024)
+  size_t smem_need = 0;
+  auto launch = [&](auto *kernel) {
+    const cudaError_t le = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)smem_need);
+    if (le == cudaSuccess) kernel<<<grid, kThreads, smem_need, stream>>>(tq, tka, tkb, a);
+    return le;
+  };
+  constexpr size_t kMaxSmem = 227 * 1024;
+  if (D == 128) {
+    smem_need = DLayout<128, 3>::alloc(max_docs, n_regions);
+    const bool three = smem_need + 1024 <= kMaxSmem;  // with the static shared memory
+    if (!three) smem_need = DLayout<128, 2>::alloc(max_docs, n_regions);
+    if (smem_need <= kMaxSmem)
+      e = three ? launch(deviation_kernel<128, 3>) : launch(deviation_kernel<128, 2>);
+  } else {
+    smem_need = DLayout<64, 3>::alloc(max_docs, n_regions);
+    const bool three = smem_need + 1024 <= kMaxSmem;  // with the static shared memory
+    if (!three) smem_need = DLayout<64, 2>::alloc(max_docs, n_regions);
+    if (smem_need <= kMaxSmem)
+      e = three ? launch(deviation_kernel<64, 3>) : launch(deviation_kernel<64, 2>);
+  }
+  if (smem_need > kMaxSmem)
     return fail(PIC_ERR_UNSUPPORTED, "pic_attention_deviation: %d documents per request do not fit the "
                 "shared-memory document table", max_docs);
-  if (D == 128) {
-    const int smem = (int)smem_need;
-    e = cudaFuncSetAttribute(deviation_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) deviation_kernel<128><<<grid, kThreads, smem, stream>>>(tq, tka, tkb, a);
-  } else {
-    const int smem = (int)smem_need;
-    e = cudaFuncSetAttribute(deviation_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) deviation_kernel<64><<<grid, kThreads, smem, stream>>>(tq, tka, tkb, a);
-  }
   if (e != cudaSuccess) return cuda_fail(e, "pic_attention_deviation smem attribute");
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "pic_attention_deviation launch");
