@@ -508,6 +508,19 @@ PIC_DEV bool mbar_wait_for(uint32_t bar, uint32_t parity, volatile int *abort, i
     }
   }
 }
+// Bounded by its limit alone, for waits that end without the abort flag.
+PIC_DEV bool mbar_wait_no_flag(uint32_t bar, uint32_t parity, int32_t *status, int detail,
+                               uint64_t limit_ns) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = globaltimer_ns();
+  for (uint32_t i = 1;; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((i & 63u) == 0 && globaltimer_ns() - t0 > limit_ns) {
+      dev_fail(status, PIC_DEV_TIMEOUT, detail);
+      return false;
+    }
+  }
+}
 // The wait every kernel of the path uses.
 PIC_DEV bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort, int32_t *status,
                        int detail) {

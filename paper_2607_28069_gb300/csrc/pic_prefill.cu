@@ -56,10 +56,12 @@ constexpr int threads_of() { return kFused ? kThreadsFused : kThreads; }
 constexpr int kWarpV = 2 + 4 * NQ;        // the V producer warp
 constexpr int kWarpRing = kWarpV + 1;     // waits for K and V on the MMA warp's behalf
 // Named barriers; 0 is __syncthreads, 1 and 2 belong to the softmax
-// warpgroups' epilogue.  On 3 + t and 5 + t the four softmax warps of query
+// warpgroups' epilogue.  On 3 + t and 7 + t the four softmax warps of query
 // tile t hand the first kPart keys' columns of P_t(j) and the rest to the MMA
-// warp; on 7 the ring warp meets it once K(j) and V(j-1) are there.
-constexpr int kNbP1 = 3, kNbP2 = 5, kNbRing = 7;
+// warp (at d = 64, where a softmax may be a tile ahead of the MMA warp, two
+// more for the odd j); on 11 the ring warp meets it once the K and V tiles of
+// its next iteration are there.
+constexpr int kNbP1 = 3, kNbP2 = 7, kNbRing = 11;
 constexpr int kPvThreads = 128 + 32;
 constexpr int kPart = 64;  // keys of a tile whose P is handed over first
 constexpr int kMaxSplits = 32;
@@ -88,8 +90,8 @@ enum {
   B_KEMPTY = B_KFULL + NSK,
   B_VFULL = B_KEMPTY + NSK,
   B_VEMPTY = B_VFULL + NSV,
-  B_SFULL = B_VEMPTY + NSV,  // one per query tile
-  B_OFINAL = B_SFULL + NQ,
+  B_SFULL = B_VEMPTY + NSV,  // NQ * (j % 2) + query tile (d = 64), query tile (d = 128)
+  B_OFINAL = B_SFULL + 2 * NQ,
   B_KROT = B_OFINAL + 1,  // rotate-on-load: this CTA's half of K(j) rotated (one arrival per rotator warp)
   B_KPEER = B_KROT + NSK,  // rotate-on-load: the cluster peer's rotated half of K(j) has landed
   B_EXIT = B_KPEER + NSK,  // rotate-on-load: the peer is done with this CTA's shared memory
@@ -203,11 +205,20 @@ struct PageSrc {
 };
 
 // One CTA = (pair of 128-row query tiles, key split, kv head, request).
-// TMEM: S_t at columns 128 t (P_t written over it as bf16), O_t at 256 + 128 t.
-// MMA order per KV tile j: PV_0(j-1), QK_0(j), PV_1(j-1), QK_1(j).  Because
-// tcgen05 MMAs of one thread complete in order, "S_t(j) is ready" implies
-// PV_t(j-1) has finished, so softmax t may rescale O_t right away, and
-// softmax 0 runs while the tensor core works on tile 1 and vice versa.
+// TMEM at d = 128: S_t at columns 128 t (P_t written over it as bf16), O_t at
+// 256 + 128 t.  MMA order per KV tile j: PV_0(j-1), QK_0(j), PV_1(j-1),
+// QK_1(j).  Because tcgen05 MMAs of one thread complete in order, "S_t(j) is
+// ready" implies PV_t(j-1) has finished, so softmax t may rescale O_t right
+// away, and softmax 0 runs while the tensor core works on tile 1 and vice versa.
+//
+// At d = 64 (kAhead) O takes half the columns and a third S buffer fits: step
+// i = 2 j + t keeps S_t(j) and P_t(j) in buffer i % 3, and the MMA order is
+// PV(i), QK(i + 3) -- into the buffer PV(i) has just read -- so S_t(j) is
+// there before softmax t is done with tile j - 1 and QK, its latency and the
+// hand-over leave the chain that bounds the period.  "PV_t(j-1) has finished"
+// is then the commit behind QK(2 j + t + 1), which only a rescale waits for.
+// (5 ragged requests of up to 9 x 1201 tokens, GQA 16/2, append included: 52.3
+// -> 45.9 us against two buffers in place; d = 128 has no columns left.)
 // Bound by the chain S -> softmax -> P -> PV of the two tiles and, on long
 // contexts, by the power limit.  The MMA warp runs converged and issues
 // through its elected lane (mma_ss): issued from a lane-0 branch that also
@@ -251,6 +262,14 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
                                           RopeParams rp) {
   using L = Layout<D>;
   constexpr int PANELS = D / 64;
+  constexpr bool kAhead = D == 64;
+  // columns of O_t: behind two S buffers, or behind three
+  constexpr uint32_t kColO = kAhead ? 384 : 256;
+  static_assert(kColO + NQ * D <= kTmemCols, "S and O fit the TMEM");
+  // the barrier S_t(j) is committed to, its parity, and the named barriers of P_t(j)
+  auto sfull = [](int t, int j) { return B_SFULL + (kAhead ? NQ * (j & 1) : 0) + t; };
+  auto sfull_parity = [](int j) -> uint32_t { return (kAhead ? j >> 1 : j) & 1; };
+  auto nb_p = [](int base, int t, int j) { return base + (kAhead ? NQ * (j & 1) : 0) + t; };
   constexpr uint32_t IDESC_QK = idesc_bf16(BM, BN, false, false);
   constexpr uint32_t IDESC_PV = idesc_bf16(BM, D, false, true);
   // K/V ring tiles are page-major: page p of a tile at p * kPageBytes.  At
@@ -602,63 +621,87 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     const MatDesc dQ = sdesc_sw128(sbase + L::kQ, 16, 1024);
     const MatDesc dK = sdesc_sw128(sbase + L::kK, 16, kGroupStride);
     const MatDesc dV = sdesc_sw128(sbase + L::kV, kPanelOff, kGroupStride);
-    for (int j = 0; j <= un; ++j) {
-      // K(j) and V(j-1) (and at first Q) are there, or a wait has failed
-      const bool go = !named_bar_or(kNbRing, 64, false);
+    // O_t += P_t(j) V(j) from the S buffer at column tS, one page of 16 keys
+    // per MMA: the first kPart keys while the softmax is still at the others
+    auto pv = [&](int t, int j, uint32_t tS, bool go) {
+      const uint32_t tO = ub + kColO + t * D;
+      const int st = j % NSV;
+      const MatDesc dv = dV.at(st * L::kTile);
+      named_bar_sync(nb_p(kNbP1, t, j), kPvThreads);
       tc_fence_after();
+      if (go)
 #pragma unroll
-      for (int t = 0; t < NQ; ++t) {
-        if (t >= u_ntile) break;
-        const uint32_t tS = ub + t * 128, tO = ub + 256 + t * 128;
-        // O_t += P_t(j-1) V(j-1), one page of 16 keys per MMA: the first
-        // kPart keys while the softmax is still at the others
-        if (j >= 1 && j - 1 < unt[t]) {
-          const int pj = j - 1, pst = pj % NSV;
-          const MatDesc dv = dV.at(pst * L::kTile);
-          named_bar_sync(kNbP1 + t, kPvThreads);
-          tc_fence_after();
-          if (go)
+        for (int kk = 0; kk < kPart / 16; ++kk)
+          mma_ts(tO, tS + kk * 8, dv.at(kk * kPageBytes), IDESC_PV, (j > 0 || kk > 0), el);
+      named_bar_sync(nb_p(kNbP2, t, j), kPvThreads);
+      tc_fence_after();
+      if (go) {
 #pragma unroll
-            for (int kk = 0; kk < kPart / 16; ++kk)
-              mma_ts(tO, tS + kk * 8, dv.at(kk * kPageBytes), IDESC_PV, (pj > 0 || kk > 0), el);
-          named_bar_sync(kNbP2 + t, kPvThreads);
-          tc_fence_after();
-          if (go) {
-#pragma unroll
-            for (int kk = kPart / 16; kk < BN / 16; ++kk)
-              mma_ts(tO, tS + kk * 8, dv.at(kk * kPageBytes), IDESC_PV, 1, el);
-            // the last tile that reads V(j-1) releases it (tile 1 reads a prefix of tile 0's range)
-            if (t == u_ntile - 1 || pj >= unt[1]) mma_commit(bar(B_VEMPTY + pst), el);
-          }
-        }
-        // S_t = Q_t K(j)^T
-        if (go && j < unt[t]) {
-          const int st = j % NSK;
-          const MatDesc dk = dK.at(st * L::kTile), dq = dQ.at(t * L::kQTile);
-#pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk)
-            mma_ss(tS, dq.at((kk >> 2) * (BM * 128) + (kk & 3) * 32),
-                   dk.at((kk >> 2) * kPanelOff + (kk & 3) * 32), IDESC_QK, kk > 0, el);
-          mma_commit(bar(B_SFULL + t), el);
-          if (t == u_ntile - 1 || j >= unt[1]) release_k(st);  // last reader of K(j)
-        }
+        for (int kk = kPart / 16; kk < BN / 16; ++kk)
+          mma_ts(tO, tS + kk * 8, dv.at(kk * kPageBytes), IDESC_PV, 1, el);
+        // the last tile that reads V(j) releases it (tile 1 reads a prefix of tile 0's range)
+        if (t == u_ntile - 1 || j >= unt[1]) mma_commit(bar(B_VEMPTY + st), el);
       }
-      // a key tile only the cluster peer uses: both halves are in this CTA's
-      // ring (its rotators are done with it, the peer's copy has landed)
-      if (kFused && go && j < un && j >= unt[0]) release_k(j % NSK);
+    };
+    // S_t = Q_t K(j)^T.  After a failed wait nothing is computed but the
+    // commit still comes: a softmax warp waits for no flag, and meets every
+    // named barrier exactly once per key tile in any case.
+    auto qk = [&](int t, int j, uint32_t tS, bool go) {
+      const int st = j % NSK;
+      const MatDesc dk = dK.at(st * L::kTile), dq = dQ.at(t * L::kQTile);
+      if (go)
+#pragma unroll
+        for (int kk = 0; kk < D / 16; ++kk)
+          mma_ss(tS, dq.at((kk >> 2) * (BM * 128) + (kk & 3) * 32),
+                 dk.at((kk >> 2) * kPanelOff + (kk & 3) * 32), IDESC_QK, kk > 0, el);
+      mma_commit(bar(sfull(t, j)), el);
+      if (go && (t == u_ntile - 1 || j >= unt[1])) release_k(st);  // last reader of K(j)
+    };
+    if constexpr (kAhead) {
+      uint32_t buf = 2;  // of step 2 j + t: (2 j + t) mod 3
+      for (int j = -2; j < un; ++j) {
+        const bool go = !named_bar_or(kNbRing, 64, false);  // K(j+2), V(j) are there
+        tc_fence_after();
+#pragma unroll
+        for (int t = 0; t < NQ; ++t) {
+          const uint32_t tS = ub + buf * 128;
+          const int ts = t ^ 1, js = j + 1 + t;  // step 2 j + t + 3
+          if (j >= 0 && j < unt[t]) pv(t, j, tS, go);
+          if (js >= 0 && js < unt[ts]) qk(ts, js, tS, go);
+          else if (js >= 0) mma_commit(bar(sfull(ts, js)), el);  // PV_t(j) is done: see the rescale
+          buf = buf == 2 ? 0 : buf + 1;
+        }
+        if (kFused && go && j + 2 < un && j + 2 >= unt[0]) release_k((j + 2) % NSK);
+      }
+    } else {
+      for (int j = 0; j <= un; ++j) {
+        const bool go = !named_bar_or(kNbRing, 64, false);  // K(j), V(j-1) are there
+        tc_fence_after();
+#pragma unroll
+        for (int t = 0; t < NQ; ++t) {
+          if (t >= u_ntile) break;
+          const uint32_t tS = ub + t * 128;
+          if (j >= 1 && j - 1 < unt[t]) pv(t, j - 1, tS, go);
+          if (j < unt[t]) qk(t, j, tS, go);
+        }
+        // a key tile only the cluster peer uses: both halves are in this CTA's
+        // ring (its rotators are done with it, the peer's copy has landed)
+        if (kFused && go && j < un && j >= unt[0]) release_k(j % NSK);
+      }
     }
     mma_commit(bar(B_OFINAL), el);
   };
   auto role_ring = [&]() {
     // ===================================================== ring warp
     // The MMA warp's waits for Q, K(j) (rotate-on-load: both halves) and
-    // V(j-1); it meets the MMA warp once per iteration.
+    // V(j - kLag); it meets the MMA warp once per iteration.
+    constexpr int kLag = kAhead ? 2 : 1;
     bool ok = true;
     auto wait = [&](int i, uint32_t parity) {
       if (ok) ok = mbar_wait(bar(i), parity, abort_flag, p.status, detail);
     };
     wait(B_Q, 0);
-    for (int j = 0; j <= n; ++j) {
+    for (int j = 0; j < n + kLag; ++j) {
       if (j < n) {
         const uint32_t par = (j / NSK) & 1;
         if constexpr (kFused) {
@@ -668,7 +711,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
           wait(B_KFULL + j % NSK, par);
         }
       }
-      if (j >= 1 && j - 1 < nt[0]) wait(B_VFULL + (j - 1) % NSV, ((j - 1) / NSV) & 1);
+      if (j >= kLag && j - kLag < nt[0]) wait(B_VFULL + (j - kLag) % NSV, ((j - kLag) / NSV) & 1);
       ok = __all_sync(0xffffffffu, ok);
       named_bar_or(kNbRing, 64, !ok);
     }
@@ -823,16 +866,25 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     const int tok = valid ? rg / p.G : 0, g = valid ? rg % p.G : 0;
     const int pos = valid ? ipos[tok] : -1;
     const uint32_t tl = tbase + ((uint32_t)(wq * 32) << 16);
-    const uint32_t tS = tl + t * 128, tO = tl + 256 + t * 128;
+    const uint32_t tO = tl + kColO + t * D;
+    uint32_t buf = t;  // S buffer: t, or (2 j + t) mod 3
     float m_used = -INFINITY, l = 0.f;
     bool ok = true;
-    int j_done = 0;  // tiles handed to the issuer
-    for (int j = 0; j < my_n; ++j, ++j_done) {
-      const int key0 = (kv_begin + j) * BN;
-      if (!__all_sync(0xffffffffu, mbar_wait(bar(B_SFULL + t), j & 1, abort_flag, p.status, detail))) {
+    // The MMA warp commits every S_t(j), also after an abort (its own waits are
+    // the ring warp's, bounded by kWaitLimitNs), so this wait looks at no flag
+    // and its longer limit only guards against MMAs that never complete; a tile
+    // of an aborted CTA is worked off like any other and its results dropped.
+    auto wait_s = [&](int i, uint32_t parity) {
+      if (!__all_sync(0xffffffffu, mbar_wait_no_flag(bar(i), parity, p.status, detail, 4 * kWaitLimitNs))) {
+        *abort_flag = 1;
         ok = false;
-        break;
       }
+    };
+    for (int j = 0; j < my_n; ++j) {
+      const int key0 = (kv_begin + j) * BN;
+      const uint32_t tS = tl + buf * 128;
+      if constexpr (kAhead) buf = buf == 0 ? 2 : buf - 1;
+      wait_s(sfull(t, j), sfull_parity(j));
       tc_fence_after();
       float s[BN];
 #pragma unroll
@@ -871,8 +923,14 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
             alpha = ex2(m_used - m_new);
             m_used = m_new;
           }
-          // O correction: PV_t(j-1) has completed (it precedes QK_t(j) in the MMA order)
+          // O correction: PV_t(j-1) has completed (it precedes QK_t(j) in the
+          // MMA order; at d = 64 the QK of step 2 j + t + 1, whose barrier is
+          // not used again before this tile's P is handed over)
           if (j > 0 && __any_sync(0xffffffffu, resc)) {
+            if constexpr (kAhead) {
+              wait_s(sfull(t ^ 1, j + t), sfull_parity(j + t));
+              tc_fence_after();
+            }
 #pragma unroll 1
             for (int c = 0; c < D / 16; ++c) {
               float o[16];
@@ -920,7 +978,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
-        named_bar_arrive(kNbP1 + t, kPvThreads);
+        named_bar_arrive(nb_p(kNbP1, t, j), kPvThreads);
 #pragma unroll
         for (int c0 = kPart; c0 < BN; c0 += 32) keys32(c0);
         f2unpack(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), l0, l1);
@@ -930,15 +988,11 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      named_bar_arrive(kNbP2 + t, kPvThreads);  // the rest of P_t(j)
-    }
-    // after an abort: meet the issuer at the barriers of the remaining tiles
-    for (; j_done < my_n; ++j_done) {
-      named_bar_sync(kNbP1 + t, kPvThreads);
-      named_bar_sync(kNbP2 + t, kPvThreads);
+      named_bar_arrive(nb_p(kNbP2, t, j), kPvThreads);  // the rest of P_t(j)
     }
     // ---- epilogue
-    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar(B_OFINAL), 0, abort_flag, p.status, detail));
+    wait_s(B_OFINAL, 0);
+    ok = __all_sync(0xffffffffu, ok && !*abort_flag);
     tc_fence_after();
     if (t < ntile && my_n == 0) {  // this tile needs none of the split's keys
       if (ok && p.num_splits > 1) {

@@ -6,7 +6,7 @@ Keys at chosen positions of later tiles are scaled up so that many rows jump by
 more than 57 in the log2 domain, in the first half, the second half, both and
 the last (masked) tile.  Reference: 64-bit softmax over the same bf16 cache and
 the same bf16 rotated queries; bound: probabilities and outputs rounded to bf16
-(2^-9 each, rows of size O(1)) and 32-bit scores of up to about 2000 (2^-24 of
+(2^-8 each, rows of size O(1)) and 32-bit scores of up to about 2000 (2^-24 of
 that, 1.2e-4, in the exponent), within the bars of the other attention tests."""
 import numpy as np
 import pytest
