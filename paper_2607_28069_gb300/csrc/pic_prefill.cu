@@ -107,7 +107,27 @@ struct Params {
   __half *part_o;  // split partials: O / l per row, fp16
   int32_t *status;
   float scale_log2;
+  int cut1, cut2;  // an unsplit grid's pair order (pair_cuts); cut1 = 0: request by request
 };
+
+// Order of an unsplit grid.  The CTAs of a request's pairs differ in length
+// where its inline tokens lie apart (spans after documents, the prefix), and
+// request by request the last ones to start may be long.  So the pairs
+// [0, cut1) of every (request, kv head) come first, then [cut1, cut2), then the
+// rest: half and quarters of the pairs, longest first, an even number each
+// (clusters of two).  The pairs of a group still start together and share their
+// K/V tiles through L2: a first group of two pairs instead of four cost 12
+// requests of 1.2k-8k keys 2%.  Request by request -> in groups, one layer: 8 x
+// 17k with spans, rotate-on-load 1219 -> 1172 us, 6 ragged requests of 10k keys
+// 171 -> 161, 8 x 16.8k at d = 64 147.5 -> 143, 12 x 8k 247 -> 243.5.  Not below
+// 4096 keys (12 x 2.5k: 122.3 -> 122.5, 12 x 1.2k: 81.8 -> 82.8), not in a single
+// wave, and not for split grids, whose CTAs are short and stay split-major.
+inline void pair_cuts(int npairs, int splits, int pages, long long heads, int *cut1, int *cut2) {
+  const bool on = splits == 1 && npairs > 4 && pages >= 256 && npairs * heads > 152 &&
+                  (npairs + 1) * heads < (1LL << 31);
+  *cut1 = on ? std::max(4, 2 * ((npairs + 2) / 4)) : 0;
+  *cut2 = on ? std::max(4, 2 * ((3 * npairs + 4) / 8)) : 0;
+}
 
 // Source of one page of 16 positions (written by fused_setup_kernel): kind as
 // PageSrc below; for kind 1 the pool row of its first position and the
@@ -304,10 +324,24 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
   // found it evicted (1.48x the algorithmic K/V read on the 4 x 139k
   // workload, 1.05x in this order).  Query tiles are counted from a
   // request's last row, so pair 0, which sees the most keys, goes first.
+  // An unsplit grid of several waves is taken in pair_cuts' order instead.
   const int npairs = (int)gridDim.x / p.num_splits;
   const int split = (int)blockIdx.x / npairs;
-  const int pair = (int)blockIdx.x % npairs;
-  const int hk = blockIdx.y, b = blockIdx.z;
+  int pair = (int)blockIdx.x % npairs;
+  int hk = blockIdx.y, b = blockIdx.z;
+  if (p.cut1 > 0) {  // unsplit: group of pairs, request, kv head, pair (see pair_cuts)
+    const unsigned heads = gridDim.y * gridDim.z;
+    const unsigned n0 = heads * p.cut1, n1 = heads * (p.cut2 - p.cut1);
+    unsigned i = blockIdx.x + npairs * (blockIdx.y + gridDim.y * blockIdx.z);
+    int p0 = 0, width = p.cut1;
+    if (i >= n0 + n1) i -= n0 + n1, p0 = p.cut2, width = npairs - p.cut2;
+    else if (i >= n0) i -= n0, p0 = p.cut1, width = p.cut2 - p.cut1;
+    pair = p0 + (int)(i % width);
+    i /= width;
+    hk = __shfl_sync(0xffffffffu, (int)(i % gridDim.y), 0);
+    b = __shfl_sync(0xffffffffu, (int)(i / gridDim.y), 0);
+    pair = __shfl_sync(0xffffffffu, pair, 0);
+  }
   const int detail = b;
 
   // ---- set-up that reads nothing the previous kernel writes: it runs before
@@ -1584,17 +1618,20 @@ extern "C" int32_t pic_prefill_plan_splits(const pic_geom_t *geom, int32_t batch
     if (sp > 1 && work * Hkv / kSms + merge > best) break;
     std::fill(sm.begin(), sm.end(), 0.0);
     std::make_heap(sm.begin(), sm.end(), std::greater<double>());
-    for (int b = 0; b < batch; ++b)
-      for (int hk = 0; hk < Hkv; ++hk)
-        for (int x = 0; x < npairs * sp; ++x) {
-          const int pr = x % npairs, split = x / npairs;
-          const int na = pair_tiles[(size_t)b * npairs + pr];
-          const int per = (na + sp - 1) / sp;
-          const int n = std::max(0, std::min(per, na - split * per));
-          std::pop_heap(sm.begin(), sm.end(), std::greater<double>());
-          sm.back() += n > 0 ? n + kCtaFixed : kCtaEmpty;
-          std::push_heap(sm.begin(), sm.end(), std::greater<double>());
-        }
+    int cuts[4] = {0, 0, 0, npairs};  // groups of pairs in launch order
+    pair_cuts(npairs, sp, (max_ctx + 15) / 16, (long long)Hkv * batch, &cuts[1], &cuts[2]);
+    for (int g = 0; g < 3; ++g)
+      for (int b = 0; b < batch; ++b)
+        for (int hk = 0; hk < Hkv; ++hk)
+          for (int split = 0; split < sp; ++split)
+            for (int pr = cuts[g]; pr < cuts[g + 1]; ++pr) {
+              const int na = pair_tiles[(size_t)b * npairs + pr];
+              const int per = (na + sp - 1) / sp;
+              const int n = std::max(0, std::min(per, na - split * per));
+              std::pop_heap(sm.begin(), sm.end(), std::greater<double>());
+              sm.back() += n > 0 ? n + kCtaFixed : kCtaEmpty;
+              std::push_heap(sm.begin(), sm.end(), std::greater<double>());
+            }
     const double cost = *std::max_element(sm.begin(), sm.end()) + (sp > 1 ? merge : 0.0);
     if (cost < best - 1e-9) {
       best = cost;
@@ -1724,7 +1761,7 @@ namespace prefill {
 
 // The attention launch (and the merge launch when the key range is split).
 template <int D, bool kFused>
-static cudaError_t launch_attention(const Plan &pl, const Params &pp, const FusedArgs &fa,
+static cudaError_t launch_attention(const Plan &pl, const Params &params, const FusedArgs &fa,
                                     const RopeParams &rp, const CUtensorMap &tq,
                                     const CUtensorMap &tk, const CUtensorMap &tv,
                                     const CUtensorMap &tkp, const CUtensorMap &tvp,
@@ -1743,11 +1780,13 @@ static cudaError_t launch_attention(const Plan &pl, const Params &pp, const Fuse
     // page sources and document cos/sin of the call, ahead of the attention
     const int page_blocks = (fa.n_pidx + 7) / 8;
     const int doc_blocks = (fa.max_docs + 256 / fa.half - 1) / (256 / fa.half);
-    e = launch_dependent(fused_setup_kernel, dim3(page_blocks + doc_blocks, pp.batch), dim3(256), 0,
-                         stream, fa, rp, pp.batch, page_blocks, pp.status);
+    e = launch_dependent(fused_setup_kernel, dim3(page_blocks + doc_blocks, params.batch), dim3(256), 0,
+                         stream, fa, rp, params.batch, page_blocks, params.status);
     if (e != cudaSuccess) return e;
   }
   const int npairs = (pl.m_tiles + NQ - 1) / NQ;
+  Params pp = params;
+  pair_cuts(npairs, pl.splits, pl.n_pidx, (long long)pp.Hkv * pp.batch, &pp.cut1, &pp.cut2);
   if constexpr (kFused) {
     // clusters of two consecutive query pairs: an even count per key split
     dim3 grid(((npairs + 1) & ~1) * pl.splits, pp.Hkv, pp.batch);
