@@ -1288,8 +1288,9 @@ struct AppendArgs {
 };
 
 template <int D>
-PIC_DEV void append_token(const AppendArgs &a, const RopeParams &rp) {
+__global__ void __launch_bounds__(256) append_kernel(AppendArgs a, RopeParams rp) {
   constexpr int HALF = D / 2, KC = D / 16, VC = D / 8;
+  pdl_entry();
   const int t = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
   const int tin = min(max(a.inline_len[b], 0), a.max_inline);
   __shared__ float2 cs[HALF];
@@ -1406,19 +1407,6 @@ PIC_DEV void append_token(const AppendArgs &a, const RopeParams &rp) {
                   ld_stream(a.v + (tok * a.Hkv + h) * D + c * 8));
     }
   }
-}
-
-// kBeside: launched right behind the relocation of a large pic_link.  An append
-// writes other slots than the relocation and reads only what the layout's
-// kernel wrote, which is complete once the relocation lets this grid launch (see
-// pdl_entry), so its CTAs work beside the relocation's last ones and wait for
-// them only before they end, which keeps completion in order: link of 6 x 20
-// documents, 3 layers 138.0 -> 133.4 us, of 8 x 16 documents, 4 layers 536.7 -> 532.6.
-template <int D, bool kBeside>
-__global__ void __launch_bounds__(256) append_kernel(AppendArgs a, RopeParams rp) {
-  if constexpr (!kBeside) pdl_entry();
-  append_token<D>(a, rp);
-  if constexpr (kBeside) pdl_entry();
 }
 
 struct Plan {
@@ -1658,7 +1646,7 @@ static pic_status_t launch_append(const char *who, const pic_geom_t *geom, const
                                   pic_stream_t stream, int32_t max_docs = 0,
                                   const int32_t *num_docs = nullptr,
                                   const int32_t *prefix_len = nullptr,
-                                  const int32_t *query_len = nullptr, bool beside = false) {
+                                  const int32_t *query_len = nullptr) {
   if ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(k_new) |
        reinterpret_cast<uintptr_t>(v_new) | reinterpret_cast<uintptr_t>(k_cache) |
        reinterpret_cast<uintptr_t>(v_cache)) & 15)
@@ -1696,9 +1684,8 @@ static pic_status_t launch_append(const char *who, const pic_geom_t *geom, const
   if (t_slots > INT32_MAX / 2 || batch > 65535)
     return fail(PIC_ERR_UNSUPPORTED, "%s: grid too large", who);
   dim3 agrid(t_slots, batch);
-  auto kernel = D == 128 ? (beside ? append_kernel<128, true> : append_kernel<128, false>)
-                         : (beside ? append_kernel<64, true> : append_kernel<64, false>);
-  cudaError_t le = launch_dependent(kernel, agrid, dim3(256), 0, stream, aa, rp);
+  cudaError_t le = D == 128 ? launch_dependent(append_kernel<128>, agrid, dim3(256), 0, stream, aa, rp)
+                            : launch_dependent(append_kernel<64>, agrid, dim3(256), 0, stream, aa, rp);
   if (le != cudaSuccess) return cuda_fail(le, "append launch");
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "append launch");
@@ -1718,7 +1705,7 @@ pic_status_t link_append(const pic_geom_t *geom, const RopeParams &rp, int32_t l
   return prefill::launch_append("pic_link", geom, rp, pl, layer, batch, max_inline, q, k_new, v_new,
                                 inline_pos, inline_len, slot_mapping, nullptr, 0, max_ctx, num_pages,
                                 k_cache, v_cache, workspace, stream, max_docs, req_num_docs,
-                                prefix_len, query_len, true);
+                                prefix_len, query_len);
 }
 
 namespace prefill {

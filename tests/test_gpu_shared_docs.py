@@ -107,3 +107,46 @@ def test_large_link_refuses_what_the_small_one_does(cuda_lib):
     assert not path.k_cache[:, pages(0)].any()
     assert not path.k_cache[:, pages(1)].any()
     assert torch.equal(path.k_cache[:, pages(2)], good[:, pages(2)])
+
+
+def test_large_links_back_to_back(cuda_lib):
+    """Large links with different prefixes, document orders and block tables,
+    one right behind the other into the same layout buffers: each link's caches
+    and packed queries against the three separate calls, bit for bit.  (A
+    launch of the chain that read the layout before its wait would find the
+    link's before.)"""
+    import paper_2607_28069_gb300 as pic
+    path = _path("pairs")
+    wl, spec = path.wl, path.wl.spec
+    gen = torch.Generator().manual_seed(5)
+    requests = []
+    for i in range(4):
+        prefix = wl.prefix_len - torch.randint(0, 3, (path.B,), generator=gen, dtype=torch.int32).cuda() * (i > 0)
+        order = torch.randperm(spec.docs_per_request, generator=gen).cuda()
+        pages = torch.randperm(wl.num_pages, generator=gen).int().cuda()
+        requests.append(dict(prefix_len=prefix, inline_len=prefix + wl.query_len,
+                             req_doc_ids=wl.req_doc_ids[:, order].contiguous(),
+                             block_table=pages[wl.block_table.long().clamp(min=0)].contiguous()))
+    kc = [torch.zeros_like(path.k_cache) for _ in requests]
+    vc = [torch.zeros_like(path.v_cache) for _ in requests]
+    ws = [torch.zeros_like(path.ws_prefill) for _ in requests]
+
+    def take(i):
+        for name, value in requests[i].items():
+            setattr(wl, name, value)
+        path.k_cache, path.v_cache, path.ws_prefill = kc[i], vc[i], ws[i]
+
+    ref = []
+    for i in range(len(requests)):
+        take(i)
+        path.compose(), path.relocate_mapped(), path.append(0)
+        ref.append((kc[i].clone(), vc[i].clone(), ws[i].clone()))
+    for _ in range(5):
+        for t in kc + vc + ws:
+            t.zero_()
+        for i in range(len(requests)):
+            take(i)
+            path.link(0)
+        for got, want in zip(zip(kc, vc, ws), ref):
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
+    assert pic.pic_device_status() == (0, 0)
