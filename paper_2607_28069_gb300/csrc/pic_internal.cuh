@@ -526,6 +526,14 @@ PIC_DEV bool mbar_wait_no_flag(uint32_t bar, uint32_t parity, int32_t *status, i
     }
   }
 }
+// One of a row of such waits: once one of them has run out, the later ones
+// return at once, so a warp that works off a loop of them is held up by the
+// limit once and not once per tile.  Called by a converged warp; `ok` is the
+// same in all its lanes.
+PIC_DEV bool mbar_wait_while(bool ok, uint32_t bar, uint32_t parity, int32_t *status, int detail,
+                             uint64_t limit_ns) {
+  return ok && __all_sync(0xffffffffu, mbar_wait_no_flag(bar, parity, status, detail, limit_ns));
+}
 // The wait every kernel of the path uses.
 PIC_DEV bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort, int32_t *status,
                        int detail) {

@@ -908,11 +908,11 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     // the ring warp's, bounded by kWaitLimitNs), so this wait looks at no flag
     // and its longer limit only guards against MMAs that never complete; a tile
     // of an aborted CTA is worked off like any other and its results dropped.
+    // After a wait that ran out the remaining tiles wait for nothing.
     auto wait_s = [&](int i, uint32_t parity) {
-      if (!__all_sync(0xffffffffu, mbar_wait_no_flag(bar(i), parity, p.status, detail, 4 * kWaitLimitNs))) {
-        *abort_flag = 1;
-        ok = false;
-      }
+      const bool was = ok;
+      ok = mbar_wait_while(ok, bar(i), parity, p.status, detail, 4 * kWaitLimitNs);
+      if (was && !ok) *abort_flag = 1;
     };
     for (int j = 0; j < my_n; ++j) {
       const int key0 = (kv_begin + j) * BN;
