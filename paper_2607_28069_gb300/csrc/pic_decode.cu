@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(kThreads)
   if (done < cw) {
     // aborted: let the loads already issued land before the ring is reused
     for (int i = done; i < min(cw, done + NSTG); ++i)
-      mbar_wait(full(i % NSTG), (i / NSTG) & 1, abort_flag, p.status, b);
+      mbar_wait_no_flag(full(i % NSTG), (i / NSTG) & 1, p.status, b, kWaitLimitNs);
   }
   // ---- reduce l over the 8 key lanes, then merge the four warps
 #pragma unroll

@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         return t < a.max_ctx ? a.slots[(size_t)b * a.max_ctx + t] : -1;
       };
       long long slot_next = load_slot(0);
+      int issued = 0;
       for (int j = 0; j < n; ++j) {
         const int st = j % NS;
         const long long slot = slot_next;
@@ -266,7 +267,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             tma_load_2d(dst + L::kTile, &tm_kb, 0, y, bar(DB_KFULL + st));
           }
         }
+        issued = j + 1;
       }
+      if (lane == 0) {  // the copies already issued land before the CTA exits, aborted or not
+        mbar_wait_no_flag(bar(DB_Q), 0, a.status, b, kWaitLimitNs);
+        for (int j = max(0, issued - NS); j < issued; ++j)
+          mbar_wait_no_flag(bar(DB_KFULL + j % NS), (j / NS) & 1, a.status, b, kWaitLimitNs);
+      }
+      __syncwarp();
     } else if (warp == kRegionWarp) {
       // ================================================ key regions
       // Lane l writes the regions of keys 4l .. 4l+3 of each tile; the bytes
@@ -448,7 +456,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid < a.n_regions && s_sum[tid] != 0.0) atomicAdd(&a.sums[(size_t)b * a.n_regions + tid], s_sum[tid]);
   if (warp == 1) {
     tc_fence_after();
-    if (r0 < row_end && n > 0 && lane == 0) mbar_wait(bar(DB_FINAL), 0, abort_flag, a.status, b);
+    if (r0 < row_end && n > 0 && lane == 0)
+      mbar_wait_no_flag(bar(DB_FINAL), 0, a.status, b, kWaitLimitNs);
     __syncwarp();
     tmem_dealloc(tbase, kTmemCols);
   }

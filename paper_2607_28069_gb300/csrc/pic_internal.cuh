@@ -513,7 +513,9 @@ PIC_DEV bool mbar_wait_for(uint32_t bar, uint32_t parity, volatile int *abort, i
     }
   }
 }
-// Bounded by its limit alone, for waits that end without the abort flag.
+// Bounded by its limit alone: for waits that end without the abort flag, and for
+// a CTA's own copies and MMAs still in flight on its way out -- after an abort
+// the flag is set, and a wait that looks at it gives up after a few polls.
 PIC_DEV bool mbar_wait_no_flag(uint32_t bar, uint32_t parity, int32_t *status, int detail,
                                uint64_t limit_ns) {
   if (mbar_try_wait(bar, parity)) return true;

@@ -486,6 +486,17 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
       }
     }
     if (!is_k && lane == 0) prefetch_tmap(&tm_v);
+    // The copies already issued land before the CTA exits, whoever aborts and
+    // when (rotate-on-load: also the cluster peer's into the same stages).
+    auto drain = [&](int issued) {
+      if (lane != 0) return;
+      if (is_k) mbar_wait_no_flag(bar(B_Q), 0, p.status, detail, kWaitLimitNs);
+      for (int j = max(0, issued - nst); j < issued; ++j) {
+        mbar_wait_no_flag(bar(b_full + j % nst), (j / nst) & 1, p.status, detail, kWaitLimitNs);
+        if (kFused && is_k)
+          mbar_wait_no_flag(bar(B_KPEER + j % nst), (j / nst) & 1, p.status, detail, kWaitLimitNs);
+      }
+    };
     if constexpr (!kFused) {
       int y_next = page_row(kv_begin);
       int issued = 0;
@@ -508,11 +519,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
         }
         issued = j + 1;
       }
-      if (lane == 0 && *abort_flag) {
-        // Let the copies already issued land before the CTA exits.
-        for (int j = max(0, issued - nst); j < issued; ++j)
-          mbar_wait(bar(b_full + j % nst), (j / nst) & 1, abort_flag, p.status, detail);
-      }
+      drain(issued);
     } else {
       // ---- rotate-on-load producers: pages from the pool or the cache as the
       // page-source table says; mixed pages row by row.  The rotators (warps
@@ -620,11 +627,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
         issue(st, kv_begin + j, s_cur);
         issued = j + 1;
       }
-      if (lane == 0 && *abort_flag) {
-        // Let the copies already issued land before the CTA exits.
-        for (int j = max(0, issued - nst); j < issued; ++j)
-          mbar_wait(bar(b_full + j % nst), (j / nst) & 1, abort_flag, p.status, detail);
-      }
+      drain(issued);
     }
   };
   auto role_issuer = [&]() {
@@ -1118,12 +1121,17 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
   __syncthreads();
   if constexpr (kFused) {
     // Leave only when the cluster peer is done too: its last copies into this
-    // CTA's ring have landed (the issuer waited for them) and it no longer
-    // reads the copies this CTA sent.  The wait is bounded even after an abort.
+    // CTA's ring have landed (the K producer waited for them) and it no longer
+    // reads the copies this CTA sent.  The wait is bounded even after an abort;
+    // a peer may then have sent pages of a tile that this CTA no longer loads
+    // and has no barrier phase for, so it stays a millisecond longer than their
+    // few microseconds.
     if (threadIdx.x == 0) {
       mbar_arrive_remote(map_to_rank(bar(B_EXIT), cpeer));
-      volatile int keep_waiting = 0;
-      mbar_wait(bar(B_EXIT), 0, &keep_waiting, p.status, detail);
+      mbar_wait_no_flag(bar(B_EXIT), 0, p.status, detail, kWaitLimitNs);
+      if (*abort_flag)
+        for (const uint64_t t0 = globaltimer_ns(); globaltimer_ns() - t0 < 1000000;) {
+        }
     }
     __syncthreads();
   }
@@ -1131,9 +1139,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
     tc_fence_after();
     if (*abort_flag && lane == 0) {
       // make sure no MMA is still running on the TMEM we are about to free
-      // (bounded by the wait limit alone: the abort flag is already set)
-      volatile int keep_waiting = 0;
-      mbar_wait(bar(B_OFINAL), 0, &keep_waiting, p.status, detail);
+      mbar_wait_no_flag(bar(B_OFINAL), 0, p.status, detail, kWaitLimitNs);
     }
     __syncwarp();
     tmem_dealloc(tbase, kTmemCols);

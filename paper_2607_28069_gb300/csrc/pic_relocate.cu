@@ -394,10 +394,8 @@ __global__ void __launch_bounds__(kThreads, 3) relocate_docs_kernel(RelocArgs a,
     }
   }
   if (!ok && tid == 0)  // aborted: let the copies already issued land before the CTA exits
-    for (long long w = u; w < min(units, u + kRing); ++w) {
-      volatile int keep_waiting = 0;
-      mbar_wait(smem_u32(&s_bar[w % kRing]), (w / kRing) & 1, &keep_waiting, a.status, b);
-    }
+    for (long long w = u; w < min(units, u + kRing); ++w)
+      mbar_wait_no_flag(smem_u32(&s_bar[w % kRing]), (w / kRing) & 1, a.status, b, kWaitLimitNs);
 }
 
 template <int D, int kTok, bool kLayerRope>

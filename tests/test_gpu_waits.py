@@ -31,6 +31,31 @@ __global__ void row_kernel(int n, unsigned long long limit_ns, int32_t *status, 
   if (threadIdx.x == 0) *got = ok;
 }
 
+// a wait of a CTA that has aborted, for a barrier that its other warp arrives on
+// only after `late_ns`
+__global__ void late_kernel(unsigned long long late_ns, unsigned long long limit_ns, int32_t *status,
+                            int *got) {
+  __shared__ __align__(8) uint64_t bar;
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&bar), 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (threadIdx.x == 32) {
+    for (const uint64_t t0 = globaltimer_ns(); globaltimer_ns() - t0 < late_ns;) {
+    }
+    mbar_arrive(smem_u32(&bar));
+  } else if (threadIdx.x == 0) {
+    *got = mbar_wait_no_flag(smem_u32(&bar), 0, status, -1, limit_ns);
+  }
+}
+
+extern "C" int late_arrival(unsigned long long late_ns, unsigned long long limit_ns, int32_t *status,
+                            int *got) {
+  late_kernel<<<1, 64>>>(late_ns, limit_ns, status, got);
+  return (int)cudaGetLastError();
+}
+
 extern "C" int row_of_waits(int n, unsigned long long limit_ns, int32_t *status, int *got) {
   row_kernel<<<1, 32>>>(n, limit_ns, status, got);
   return (int)cudaGetLastError();
@@ -53,6 +78,15 @@ def waits(cuda_lib, tmp_path_factory):
 def _ints(n):
     t = torch.zeros(n, dtype=torch.int32, device="cuda")
     return t, ctypes.c_void_p(t.data_ptr())
+
+
+def test_a_wait_on_the_way_out_waits(waits):
+    """What an aborted CTA waits for arrives 200 ms late, and is waited for."""
+    status, sp = _ints(2)
+    got, gp = _ints(1)
+    assert waits.late_arrival(ctypes.c_uint64(200_000_000), ctypes.c_uint64(2_000_000_000), sp, gp) == 0
+    torch.cuda.synchronize()
+    assert got.item() == 1 and status.tolist() == [0, 0]
 
 
 def test_a_row_of_waits_runs_out_once(waits):

@@ -1,4 +1,6 @@
-"""Programmatic dependent launches (no GPU): a kernel that calls pdl_entry calls it
+"""Order of waits in the kernels' sources (no GPU).
+
+Programmatic dependent launches: a kernel that calls pdl_entry calls it
 first and unconditionally.  Only a grid's own wait makes earlier kernels' writes
 visible to it, so nothing may be read ahead of it, and a kernel whose trigger
 came ahead of its wait would let its successor start too early."""
@@ -20,3 +22,13 @@ def test_kernels_wait_before_anything_else():
             assert all(re.match(r"(constexpr|using|static_assert)\b", s) for s in ahead), (path, ahead)
             seen += 1
     assert seen >= 6
+
+
+def test_waits_on_the_way_out_look_at_no_abort_flag():
+    """An aborted CTA waits for its copies and MMAs in flight before it exits; a
+    wait that takes the abort flag, which is set by then, gives up at once."""
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        text = open(path).read()
+        for m in re.finditer(r"if \([^{;]*\*abort_flag\)|// aborted:|if \(r0 < row_end && n > 0 && lane == 0\)", text):
+            for wait in re.findall(r"\bmbar_wait\w*\([^;]*;", text[m.end():m.end() + 500].split("\n  }\n")[0]):
+                assert wait.startswith("mbar_wait_no_flag("), (path, wait)
