@@ -9,6 +9,7 @@
 //
 // A tensor argument may also be a tuple (tensor, i) or (tensor, i, j): the
 // sub-tensor tensor[i] or tensor[i, j], without creating a Python object for it.
+// With a list or tuple of tensors in the tensor's place, i picks one of them.
 #include <Python.h>
 
 #include <ATen/core/Tensor.h>
@@ -79,6 +80,7 @@ struct View {
   }
   bool contiguous() const {
     if (skip == 0) return t->is_contiguous();
+    if (numel() == 0) return true;
     int64_t stride = 1;
     for (int64_t d = t->dim() - 1; d >= skip; --d) {
       if (t->size(d) != 1 && t->stride(d) != stride) return false;
@@ -92,21 +94,26 @@ struct View {
 View view_of(PyObject *o, const char *name) {
   View w;
   if (o == Py_None) return w;
-  PyObject *base = PyTuple_CheckExact(o) && PyTuple_GET_SIZE(o) > 0 ? PyTuple_GET_ITEM(o, 0) : o;
+  const bool indexed = PyTuple_CheckExact(o) && PyTuple_GET_SIZE(o) > 0;
+  PyObject *base = indexed ? PyTuple_GET_ITEM(o, 0) : o;
   if (base == Py_None) return w;
+  const Py_ssize_t n = indexed ? PyTuple_GET_SIZE(o) : 1;
+  Py_ssize_t i = 1;
+  auto index = [&](int64_t size) {
+    long long at = PyLong_AsLongLong(PyTuple_GET_ITEM(o, i++));
+    if (PyErr_Occurred()) throw PyErrorSet();
+    if (at < 0) at += size;
+    if (at < 0 || at >= size) raise(PyExc_IndexError, "%s: index out of range%s", name);
+    return (int64_t)at;
+  };
+  if (n > 1 && (PyList_Check(base) || PyTuple_Check(base)))  // (list, i, ...): the list keeps its item
+    base = PySequence_Fast_GET_ITEM(base, index(PySequence_Fast_GET_SIZE(base)));
   if (!THPVariable_Check(base)) raise(PyExc_TypeError, "%s must be a tensor%s", name);
   w.t = &THPVariable_Unpack(base);
-  if (base != o) {
-    w.skip = PyTuple_GET_SIZE(o) - 1;
-    if (w.skip > w.t->dim()) raise(PyExc_IndexError, "%s: too many indices%s", name);
-    for (int64_t d = 0; d < w.skip; ++d) {
-      long long at = PyLong_AsLongLong(PyTuple_GET_ITEM(o, d + 1));
-      if (PyErr_Occurred()) throw PyErrorSet();
-      if (at < 0) at += w.t->size(d);
-      if (at < 0 || at >= w.t->size(d)) raise(PyExc_IndexError, "%s: index out of range%s", name);
-      w.offset += at * w.t->stride(d) * (int64_t)w.t->element_size();
-    }
-  }
+  w.skip = n - i;
+  if (w.skip > w.t->dim()) raise(PyExc_IndexError, "%s: too many indices%s", name);
+  for (int64_t d = 0; d < w.skip; ++d)
+    w.offset += index(w.t->size(d)) * w.t->stride(d) * (int64_t)w.t->element_size();
   return w;
 }
 
@@ -528,7 +535,8 @@ PyObject *copy_async(PyObject *, PyObject *const *v, Py_ssize_t n) {
 }
 
 // Copies for a served pass: `bytes` bytes at the same byte offset of dst and
-// src, by the library's copy kernel or (engine) by a copy engine.
+// src, or (negative) the whole of two tensors of one shape, by the library's
+// copy kernel or (engine) by a copy engine.
 PyObject *copy_range(PyObject *, PyObject *const *v, Py_ssize_t n) {
   return guarded(v, n, [](Args &a) {
     View w[2];
@@ -540,22 +548,28 @@ PyObject *copy_range(PyObject *, PyObject *const *v, Py_ssize_t n) {
       if (!w[i].t->is_cuda() && !w[i].t->is_pinned())
         raise(PyExc_ValueError, "%s must be a CUDA tensor or pinned host memory%s", names[i]);
     }
+    if (w[0].t->scalar_type() != w[1].t->scalar_type() || w[0].dim() != w[1].dim())
+      raise(PyExc_ValueError, "dst and src differ in dtype or in dimensions%s%s", "");
     const int64_t offset = a.integer();
     int64_t bytes = a.integer();
     const bool engine = a.integer() != 0;
     const int64_t have = std::min(w[0].numel() * (int64_t)w[0].t->element_size(),
                                   w[1].numel() * (int64_t)w[1].t->element_size());
-    if (bytes < 0) bytes = have - offset;  // the rest
+    if (bytes < 0) {
+      for (int64_t d = 0; d < w[0].dim(); ++d)
+        if (w[0].size(d) != w[1].size(d)) raise(PyExc_ValueError, "dst and src differ in shape%s%s", "");
+      bytes = have - offset;
+    }
     if (offset < 0 || bytes < 0 || offset + bytes > have)
       raise(PyExc_ValueError, "copy range outside dst or src%s%s", "");
     char *d = static_cast<char *>(w[0].data()) + offset;
     const char *src = static_cast<const char *>(w[1].data()) + offset;
     const pic_stream_t s = stream_of(a.next());
-    return unlocked([&]() -> int {
-      if (!engine) return pic_copy_async(d, src, (size_t)bytes, s);
-      return cudaMemcpyAsync(d, src, (size_t)bytes, cudaMemcpyDefault, s) == cudaSuccess
-                 ? PIC_OK : PIC_ERR_CUDA;
-    });
+    if (!engine) return unlocked([&]() -> int { return pic_copy_async(d, src, (size_t)bytes, s); });
+    const cudaError_t e = (cudaError_t)unlocked(
+        [&]() -> int { return cudaMemcpyAsync(d, src, (size_t)bytes, cudaMemcpyDefault, s); });
+    if (e != cudaSuccess) raise(PyExc_RuntimeError, "copy failed: %s%s", cudaGetErrorString(e));
+    return (int)PIC_OK;
   });
 }
 

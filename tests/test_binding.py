@@ -64,3 +64,51 @@ def test_sub_tensors_as_tuples(cuda_lib):
         pic.pic_copy_async(dst, (src.transpose(1, 2), 0))
     with pytest.raises(ValueError, match="differ in size"):
         pic.pic_copy_async(dst, (src, 0))
+
+
+@pytest.mark.gpu
+def test_served_pass_host_buffers(cuda_lib):
+    """served_pass takes the outputs' host buffer as one tensor or as a list of
+    one per layer, and refuses buffers of another shape or type."""
+    from paper_2607_28069_gb300.pipeline import CacheHitPath
+    from paper_2607_28069_gb300.workloads import custom_spec, generate
+    spec = custom_spec(name="served_forms", layers=3, q_heads=8, kv_heads=2, head_dim=64, rope_base=1e4,
+                       batch=2, pool_docs=4, docs_per_request=3, doc_len=(20, 90), prefix_len=(3, 17),
+                       query_len=11)
+    path = CacheHitPath(generate(spec, device="cuda", gen_device="cuda"))
+    host = path.pack_request_inputs()
+    up, down = torch.cuda.Stream(), torch.cuda.Stream()
+    path.out.zero_()
+    out = torch.zeros(path.out.shape, dtype=path.out.dtype, pin_memory=True)
+    path.served_pass(host, out, up, down)
+    torch.cuda.synchronize()
+    per_layer = [torch.zeros(path.out.shape[1:], dtype=path.out.dtype, pin_memory=True) for _ in range(3)]
+    path.served_pass(host, per_layer, up, down)
+    torch.cuda.synchronize()
+    assert out.any() and torch.equal(torch.stack(per_layer), out)
+    B, T = path.out.shape[1:3]
+    for bad in (torch.zeros((3, B, T - 1) + path.out.shape[3:], dtype=path.out.dtype, pin_memory=True),
+                torch.zeros(path.out.shape, dtype=torch.float16, pin_memory=True)):
+        with pytest.raises(ValueError):
+            path.served_pass(host, bad, up, down)
+        torch.cuda.synchronize()
+    for bad in (host[:-512], host.view(torch.int32), host.view(2, -1)):
+        with pytest.raises(ValueError):
+            path.served_pass(bad, out, up, down)
+        torch.cuda.synchronize()
+    with pytest.raises(TypeError):
+        path.served_pass(host, ["no tensor"] * 3, up, down)
+    torch.cuda.synchronize()
+    assert pic.pic_device_status() == (0, 0)
+
+
+@pytest.mark.gpu
+def test_one_of_a_list_as_a_tuple(cuda_lib):
+    src = [torch.arange(64, dtype=torch.int32, device="cuda").view(2, 32) + 100 * i for i in range(3)]
+    dst = torch.zeros(32, dtype=torch.int32, device="cuda")
+    for i, j in ((0, 0), (2, 1), (-1, 0)):
+        pic.pic_copy_async(dst, (src, i, j))
+        assert torch.equal(dst, src[i][j])
+    for at in ((3, 0), (0, 2), (0, 0, 0, 0)):
+        with pytest.raises(IndexError):
+            pic.pic_copy_async(dst, (src, *at))
