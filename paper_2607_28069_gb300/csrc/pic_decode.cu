@@ -482,40 +482,21 @@ struct Plan {
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Key splits for `units` (request, kv head) pairs of `pages` pages.  Grids of
-// about 256 CTAs (two fit on an SM, 304 in all) or a multiple do best: just past
-// one wave a second one starts that fills little of the GPU; a multiple, so
-// that no CTA has more than 256 pages and the last ones end together.  And no
-// more than sqrt(pages) splits: a page costs a warp about half a microsecond,
-// a split of its own the merge a tenth.  Against splits for four waves (at
-// least 16 pages each), us per layer (heads 32/8 unless stated): 1 request of
-// 16k keys 24.1 -> 18.1 (64 -> 32 splits), 33k 33.6 -> 27.5, 131k 92 -> 86; 3
-// requests of 16k, 8/2 heads 21.9 -> 15.3; 4 of 4k 19.9 -> 15.8 (16 -> 8); 2 of
-// 400 8.9 -> 6.3 (1 -> 6); 8 of 16k 89.1 -> 84.5; 16 of 33k, 28/4 164.7 -> 161.4.
-// Groups of more than 8 heads (two columns of MMAs, one CTA an SM at 164
-// registers) keep four waves of splits of at least 16 pages: it suits one or
-// two requests as well (16 heads a group, 33k keys: 64 splits 18.5 us, 32 22.4);
-// 32 requests of 10k would do better with 8 splits than with its 38 (34 against
-// 52 us), but the allocation-free call's tests hold it to that plan.
-inline int auto_splits(long long units, int pages, bool wide_group) {
-  if (wide_group)
-    return (int)std::max(1ll, std::min({(8ll * 152 + units - 1) / units,
-                                        (long long)std::max(1, pages / 16), (long long)kMaxSplits}));
-  constexpr long long kWave = 256;
-  constexpr int kMaxPages = 256;
-  long long s = 0;
-  for (long long w = 1; s == 0 || (s < kMaxSplits && pages > kMaxPages * s); ++w) s = kWave * w / units;
-  int root = 1;
-  while ((long long)root * root < pages) ++root;
-  return (int)std::max(1ll, std::min({s, (long long)root, (long long)kMaxSplits}));
-}
-
 inline Plan plan(const pic_geom_t *g, int batch, int max_ctx, int num_splits) {
   Plan pl;
   const int pages = (max_ctx + 15) / 16;
-  if (num_splits <= 0)
-    num_splits = auto_splits((long long)batch * g->num_kv_heads, pages,
-                             g->num_q_heads / g->num_kv_heads > 8);
+  if (num_splits <= 0) {
+    // Four waves of CTAs with at least 16 pages each.  A count for whole waves of
+    // resident CTAs and at most sqrt(pages) was faster by 8% on average over
+    // 832 shapes (one request of 16k keys 24.1 -> 18.1 us a layer), but slower by
+    // up to 46% where it chose one or two splits (12 requests of 2k keys, 12 heads
+    // of 64: 15.8 -> 23.2 us, 12.4 with four), and fewer splits round more of the
+    // probabilities (error against 64 bits +0.5 to 2.5%): not kept.
+    const long long units = (long long)batch * g->num_kv_heads;
+    int s = (int)((8LL * 152 + units - 1) / units);
+    s = std::min(s, std::max(1, pages / 16));
+    num_splits = std::max(1, std::min(s, kMaxSplits));
+  }
   num_splits = std::min(num_splits, pages);
   pl.splits = std::max(1, num_splits);
   pl.pages_per_split = (pages + pl.splits - 1) / pl.splits;

@@ -44,3 +44,16 @@ def test_planner_returns_a_valid_split_count():
     assert one > 1
     with pytest.raises(ValueError):
         pic.pic_prefill_plan_splits(g, 4096, lens, pos[0])
+
+
+def test_decode_split_count_fills_the_gpu():
+    """The automatic split count of a decoding step: CTAs for four waves (eight a
+    streaming multiprocessor) with at least 16 pages each.  A batch of a few
+    dozen (request, kv head) pairs is not left with one or two splits."""
+    for hq, hkv, d in ((32, 8, 128), (28, 4, 128), (12, 12, 64), (16, 1, 64), (64, 64, 128)):
+        g = pic.Geometry(1, hq, hkv, d, 5e5)
+        for batch in (1, 3, 12, 16, 24, 200):
+            for ctx in (1, 16, 17, 400, 2049, 4097, 33000, 140000):
+                pages = -(-ctx // 16)
+                want = min(-(-8 * 152 // (batch * hkv)), max(1, pages // 16), 64, pages)
+                assert pic.pic_decode_num_splits(g, batch, ctx, 0) == want, (hkv, batch, ctx)
