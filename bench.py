@@ -481,6 +481,12 @@ def main_gpu(args, rank, world):
     flush = torch.empty(max(2 * l2, 256 << 20), dtype=torch.uint8, device=dev)
     sleep_cycles = int(2e9 * max(50e-6, 5e-6 * len(graphs)))
 
+    def launches_of(fn):
+        """Kernels of the library that one call launches."""
+        before = pic.pic_launch_count()
+        fn()
+        return pic.pic_launch_count() - before
+
     def pass_step():
         """Flush L2, then one pass with no timing nodes inside; returns ms."""
         flush.zero_()
@@ -562,9 +568,7 @@ def main_gpu(args, rank, world):
                       "tflops": work["attend_flops"] / (per_step["attend"] * 1e9)},
     }
     rows["a2_a3_relocate"]["frac_hbm"] = rows["a2_a3_relocate"]["gbs"] / peaks["hbm_gbs"]
-    # pic_link: one launch, or three when its relocation moves 128 MB or more
-    link_launches = 3 if 8.0 * spec.batch * path.max_ctx * spec.kv_heads * spec.head_dim * L >= 128e6 \
-        else 1
+    link_launches = launches_of(lambda: path.link(0))  # one, or three (large links)
     if link_ms:
         lms = sum(link_ms) / len(link_ms)
         link_bytes = work["relocate_bytes"] + work["append_bytes"] / L
@@ -595,9 +599,7 @@ def main_gpu(args, rank, world):
         dms = sum(dts) / len(dts)
         rows["a6_decode"] = {
             "ms": dms, "splits": dsplits,
-            # append and attention; the merge of more splits than a cluster takes
-            "launches": L * (2 if dsplits > 16 or dsplits * spec.kv_heads * spec.batch > 304
-                             else 1),
+            "launches": L * launches_of(lambda: path.decode(0, 0)),
             "bytes": work["decode_bytes"], "gbs": work["decode_bytes"] / (dms * 1e6),
             "tok_s": spec.batch / (dms / 1e3)}
         rows["a6_decode"]["frac_hbm"] = rows["a6_decode"]["gbs"] / peaks["hbm_gbs"]

@@ -102,6 +102,14 @@ int32_t pic_abi_version(void);
 const char *pic_last_error(void);
 
 /*
+ * pic_launch_count -- kernels that the calls of this thread have launched so
+ * far, copies by copy engines and memsets not counted: how many launches a
+ * call took is the difference around it (several entry points choose between
+ * forms with one, two or three).
+ */
+int64_t pic_launch_count(void);
+
+/*
  * pic_device_status -- synchronise `stream`, then read and clear the status
  * word of the current device.  *code receives a PIC_DEV_* value, *detail the
  * request (or split) index of the first failure.  Returns PIC_ERR_DEVICE when

@@ -17,8 +17,8 @@ from typing import Optional
 import torch
 
 __all__ = [
-    "Geometry", "load", "lib_path", "pic_abi_version", "pic_compose", "pic_relocate",
-    "pic_relocate_mapped", "pic_link",
+    "Geometry", "load", "lib_path", "pic_abi_version", "pic_launch_count", "pic_compose",
+    "pic_relocate", "pic_relocate_mapped", "pic_link",
     "pic_attention_deviation", "pic_copy_async", "pic_launch_probe", "pic_wait_probe",
     "pic_append_inline", "pic_attend_prefill", "pic_attend_prefill_fused",
     "pic_prefill_workspace_size", "pic_prefill_fused_workspace_size",
@@ -38,7 +38,8 @@ ROPE_INTERLEAVED = 1
 
 # Every symbol include/pic.h declares.
 EXPORTED_SYMBOLS = (
-    "pic_abi_version", "pic_last_error", "pic_device_status", "pic_compose", "pic_relocate",
+    "pic_abi_version", "pic_last_error", "pic_launch_count", "pic_device_status", "pic_compose",
+    "pic_relocate",
     "pic_relocate_mapped", "pic_link", "pic_attention_deviation", "pic_prefill_workspace_size",
     "pic_prefill_fused_workspace_size", "pic_prefill_num_splits", "pic_prefill_plan_splits",
     "pic_append_inline",
@@ -115,6 +116,7 @@ def load():
     sig = {
         "pic_abi_version": (I32, []),
         "pic_last_error": (ctypes.c_char_p, []),
+        "pic_launch_count": (I64, []),
         "pic_device_status": (I32, [P, P, P]),
         "pic_copy_async": (I32, [P, P, SZ, P]),
         "pic_launch_probe": (I32, [I32, P, P, P, P]),
@@ -195,6 +197,11 @@ bf16, i32, i64, f32 = torch.bfloat16, torch.int32, torch.int64, torch.float32
 
 def pic_abi_version() -> int:
     return load().pic_abi_version()
+
+
+def pic_launch_count() -> int:
+    """Kernels that this thread's calls have launched so far."""
+    return load().pic_launch_count()
 
 
 def pic_device_status(stream=None):

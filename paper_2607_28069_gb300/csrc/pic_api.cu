@@ -26,6 +26,13 @@ pic_status_t cuda_fail(cudaError_t e, const char *what) {
   return fail(PIC_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+static thread_local int64_t t_launches = 0;
+
+cudaError_t counted(cudaError_t launch) {
+  if (launch == cudaSuccess) ++t_launches;
+  return launch;
+}
+
 void *device_address(const void *p) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
@@ -226,6 +233,8 @@ extern "C" {
 int32_t pic_abi_version(void) { return PIC_ABI_VERSION; }
 
 const char *pic_last_error(void) { return pic::t_last_error; }
+
+int64_t pic_launch_count(void) { return pic::t_launches; }
 
 pic_status_t pic_device_status(pic_stream_t stream, int32_t *code, int32_t *detail) {
   int32_t *p = pic::device_status_ptr();

@@ -80,7 +80,7 @@ extern "C" pic_status_t pic_wait_probe(int32_t arrive, int64_t limit_ns, pic_str
   int32_t *status = device_status_ptr();
   if (!status) return fail(PIC_ERR_CUDA, "pic_wait_probe: no device status word");
   wait_probe_kernel<<<1, 32, 0, stream>>>(arrive != 0, (uint64_t)limit_ns, status);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = counted(cudaGetLastError());
   return e == cudaSuccess ? PIC_OK : cuda_fail(e, "pic_wait_probe launch");
 }
 
@@ -136,6 +136,6 @@ extern "C" pic_status_t pic_copy_async(void *dst, const void *src, size_t bytes,
   copy_kernel<<<(unsigned)blocks, kCopyThreads, 0, stream>>>(
       static_cast<uint4 *>(d), static_cast<const uint4 *>(s), n16,
       static_cast<uint8_t *>(d) + n16 * 16, static_cast<const uint8_t *>(s) + n16 * 16, tail);
-  e = cudaGetLastError();
+  e = counted(cudaGetLastError());
   return e == cudaSuccess ? PIC_OK : cuda_fail(e, "pic_copy_async launch");
 }

@@ -19,9 +19,9 @@
 //     of the O^T += V^T P^T MMA in registers with movmatrix.  The four warps'
 //     states are merged through shared memory at the end.
 //  2. decode_combine_kernel (only with several splits): log-sum-exp merge.
-//     A grid that fits the GPU at once and has at most 16 splits runs them as
-//     a thread-block cluster instead and merges through distributed shared
-//     memory, with no second launch.
+//     4 to 16 splits run as a thread-block cluster instead, where the GPU
+//     holds all of them at once, and merge through distributed shared memory,
+//     with no second launch.
 #include <algorithm>
 #include <mutex>
 
@@ -34,13 +34,18 @@ constexpr int kWarps = 4;
 constexpr int kThreads = 32 * kWarps;
 constexpr int NSTG = 3;
 constexpr int kMaxSplits = 64;
-constexpr int kMaxCluster = 16;  // splits of one (request, kv head) merged in a cluster
-// A grid of up to this many CTAs (two an SM) runs its splits as clusters, us per
-// layer against the merge launch: one request, 32/8 heads, 1k keys 6.42 and
-// 7.02, 128 keys 5.65 and 5.96, four of 4k 15.8 and 16.8; two of 1k, 28/4 6.75
-// and 7.37; d = 64 5.89 and 6.53.  (With the append as a launch of its own and
-// the merge launch: 10.5, 8.1, 22.0.)
-constexpr long long kClusterCtas = 304;
+// The splits of one (request, kv head) run as a cluster, merged through
+// distributed shared memory, where there are 4 to 16 of them, the groups have up
+// to 8 query heads, and the GPU holds all clusters at once (use_cluster).  us
+// per layer against the merge launch: one request, 8/2 heads, 400 keys, 16 splits
+// 5.27 and 6.67; over 1700 such shapes 0.96 of its time on average.  Clusters
+// that wait for others to end take 1.34 to 1.88 times as long as CTAs with the
+// merge launch, because a cluster needs its SMs in one GPC at once (14 clusters
+// of 16 fit at d = 128, 224 CTAs of the 304 that fit without); two or three
+// splits gain nothing (1.00 to 1.02), groups of more than 8 heads lose (1.01 to
+// 1.17, at four splits 1.05).
+constexpr int kMinCluster = 4, kMaxCluster = 16;
+constexpr long long kClusterCtas = 304;  // two CTAs an SM; larger grids are not launch-bound
 
 template <int D>
 struct Layout {
@@ -511,18 +516,84 @@ inline Plan plan(const pic_geom_t *g, int batch, int max_ctx, int num_splits) {
   return pl;
 }
 
-template <int D, int NT>
-cudaError_t launch_attn(dim3 grid, bool cluster, cudaStream_t stream, const CUtensorMap &tk,
-                        const CUtensorMap &tv, const Params &pp, const RopeParams &rp) {
-  const int smem = Layout<D>::kAlloc;
-  auto *kernel = cluster ? decode_attn_kernel<D, NT, true> : decode_attn_kernel<D, NT, false>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess && cluster && grid.x > 8)
+template <int D, int NT, bool kCluster>
+cudaError_t allow_attn() {
+  auto *kernel = decode_attn_kernel<D, NT, kCluster>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       Layout<D>::kAlloc);
+  if (kCluster && e == cudaSuccess)  // more than 8 CTAs
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return e;
+}
+
+template <int D, int NT>
+cudaError_t launch_attn(dim3 grid, cudaStream_t stream, const CUtensorMap &tk, const CUtensorMap &tv,
+                        const Params &pp, const RopeParams &rp) {
+  const cudaError_t e = allow_attn<D, NT, false>();
   if (e != cudaSuccess) return e;
-  return cluster ? launch_dependent_cluster(kernel, grid, dim3(kThreads), smem, stream, (int)grid.x,
-                                            tk, tv, pp, rp)
-                 : launch_dependent(kernel, grid, dim3(kThreads), smem, stream, tk, tv, pp, rp);
+  return launch_dependent(decode_attn_kernel<D, NT, false>, grid, dim3(kThreads), Layout<D>::kAlloc,
+                          stream, tk, tv, pp, rp);
+}
+
+template <int D>
+cudaError_t launch_attn_cluster(dim3 grid, cudaStream_t stream, const CUtensorMap &tk,
+                                const CUtensorMap &tv, const Params &pp, const RopeParams &rp) {
+  const cudaError_t e = allow_attn<D, 1, true>();
+  if (e != cudaSuccess) return e;
+  return launch_dependent_cluster(decode_attn_kernel<D, 1, true>, grid, dim3(kThreads),
+                                  Layout<D>::kAlloc, stream, (int)grid.x, tk, tv, pp, rp);
+}
+
+// Clusters of `splits` CTAs that the current device holds at once; 0 also where
+// it places none (a partition with few SMs a GPC) or does not say.  Asked once
+// per device context and size: the answer takes the runtime 1.3 us.
+template <int D>
+int resident_clusters(int splits) {
+  constexpr int kMaxDev = 64;
+  struct Known {
+    unsigned long long ctx;
+    int count[kMaxCluster + 1];  // -1: not asked yet
+  };
+  static Known known[kMaxDev];
+  static std::mutex mu;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return 0;
+  const unsigned long long id = current_context_id();
+  std::lock_guard<std::mutex> lk(mu);
+  Known &k = known[dev];
+  if (id == 0 || id != k.ctx) {
+    std::fill(k.count, k.count + kMaxCluster + 1, -1);
+    k.ctx = id;
+  }
+  if (k.count[splits] < 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(splits);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Layout<D>::kAlloc;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)splits;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    cudaError_t e = allow_attn<D, 1, true>();
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveClusters(&n, decode_attn_kernel<D, 1, true>, &cfg);
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // clear the error the failed query recorded
+      n = 0;
+    }
+    k.count[splits] = n;
+  }
+  return k.count[splits];
+}
+
+inline bool use_cluster(int D, int group, int splits, long long heads) {
+  if (group > 8 || splits < kMinCluster || splits > kMaxCluster || splits * heads > kClusterCtas)
+    return false;
+  return heads <= (D == 128 ? resident_clusters<128>(splits) : resident_clusters<64>(splits));
 }
 
 }  // namespace decode
@@ -627,14 +698,16 @@ static pic_status_t launch_step(const char *who, const pic_geom_t *geom, const R
 
   dim3 grid(pl.splits, Hkv, batch);
   cudaError_t e;
-  const bool cluster = pl.splits > 1 && pl.splits <= kMaxCluster &&
-                       (long long)pl.splits * Hkv * batch <= kClusterCtas;
-  if (D == 128)
-    e = G <= 8 ? launch_attn<128, 1>(grid, cluster, stream, tk, tv, pp, rp)
-               : launch_attn<128, 2>(grid, cluster, stream, tk, tv, pp, rp);
+  const bool cluster = use_cluster(D, G, pl.splits, (long long)Hkv * batch);
+  if (cluster)
+    e = D == 128 ? launch_attn_cluster<128>(grid, stream, tk, tv, pp, rp)
+                 : launch_attn_cluster<64>(grid, stream, tk, tv, pp, rp);
+  else if (D == 128)
+    e = G <= 8 ? launch_attn<128, 1>(grid, stream, tk, tv, pp, rp)
+               : launch_attn<128, 2>(grid, stream, tk, tv, pp, rp);
   else
-    e = G <= 8 ? launch_attn<64, 1>(grid, cluster, stream, tk, tv, pp, rp)
-               : launch_attn<64, 2>(grid, cluster, stream, tk, tv, pp, rp);
+    e = G <= 8 ? launch_attn<64, 1>(grid, stream, tk, tv, pp, rp)
+               : launch_attn<64, 2>(grid, stream, tk, tv, pp, rp);
   if (e != cudaSuccess) return cuda_fail(e, "decode attention launch");
   if (pl.splits > 1 && !cluster) {
     dim3 cgrid(geom->num_q_heads, batch);

@@ -594,7 +594,7 @@ extern "C" pic_status_t pic_attention_deviation(
     return fail(PIC_ERR_UNSUPPORTED, "pic_attention_deviation: %d documents per request do not fit the "
                 "shared-memory document table", max_docs);
   if (e != cudaSuccess) return cuda_fail(e, "pic_attention_deviation smem attribute");
-  e = cudaGetLastError();
+  e = counted(cudaGetLastError());
   if (e != cudaSuccess) return cuda_fail(e, "pic_attention_deviation launch");
   return PIC_OK;
 }

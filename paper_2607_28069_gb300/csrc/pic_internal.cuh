@@ -34,6 +34,8 @@ int32_t *device_status_ptr();
 // none or the driver cannot say): device addresses of module variables are
 // valid for one context, and a device reset replaces it.
 unsigned long long current_context_id();
+// Counts a kernel launch of the calling thread (pic_launch_count) if it went out.
+cudaError_t counted(cudaError_t launch);
 // Validates the geometry and fills theta[0..d/2) (fp64 frequencies).
 pic_status_t check_geom(const pic_geom_t *g, double *theta);
 
@@ -383,7 +385,7 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+  return counted(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
 }
 // The same, with the grid in clusters of `cluster_x` consecutive CTAs along x.
 template <typename... KArgs, typename... Args>
@@ -404,7 +406,7 @@ inline cudaError_t launch_dependent_cluster(void (*kernel)(KArgs...), dim3 grid,
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+  return counted(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
 }
 
 // ---- thread-block clusters

@@ -1486,9 +1486,9 @@ static cudaError_t launch_combine(long long rows, const Params &pp, cudaStream_t
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (U == 2) return cudaLaunchKernelEx(&cfg, combine_kernel<D, 2, 4>, pp);
-  if (U == 4) return cudaLaunchKernelEx(&cfg, combine_kernel<D, 4, 2>, pp);
-  return cudaLaunchKernelEx(&cfg, combine_kernel<D, 8, 1>, pp);
+  if (U == 2) return counted(cudaLaunchKernelEx(&cfg, combine_kernel<D, 2, 4>, pp));
+  if (U == 4) return counted(cudaLaunchKernelEx(&cfg, combine_kernel<D, 4, 2>, pp));
+  return counted(cudaLaunchKernelEx(&cfg, combine_kernel<D, 8, 1>, pp));
 }
 }  // namespace prefill
 }  // namespace pic
