@@ -1566,6 +1566,17 @@ extern "C" int32_t pic_prefill_num_splits(const pic_geom_t *geom, int32_t batch,
 // before); with spans 899 and 999 / 1018 / 1037 (3 before), rotate-on-load 1174
 // and 1300; 2 requests of 4k 28.1 with 4, 28.9 with 3; 4 of 8k, 16/2 heads of
 // 64, 30.7 with 4, 34.6 with 3; 4 of 139k 2886 with 1, 2832-2874 with 4 to 10.
+//
+// The count serves rotate-on-load as well, whose CTAs come in clusters of two
+// that both stream the upper pair's key tiles: a lower pair that is short in the
+// materialised grid takes as long as the upper one there.  So a count beyond the
+// library's own is taken only if a grid of such clusters does not take longer
+// with it either: 4 requests of 1k keys, 16 query tokens, 32/8 heads: 2 splits,
+// not 3 (rotate-on-load 32.4 us and 38.4; materialised 22 and 20); 8 of 1k, one
+// query token, 28/4 heads: 2, not 3 (34.0 and 40.2); 26 of 1164 shapes were up to
+// 19% slower.  And it has to win by more than the model is off: one request of 1k
+// keys, 512 query tokens, 16/2 heads of 64, 5 splits 3% under 4 by the model, 4%
+// over it measured.
 extern "C" int32_t pic_prefill_plan_splits(const pic_geom_t *geom, int32_t batch,
                                            int32_t max_inline, int32_t max_ctx,
                                            const int32_t *inline_len, const int32_t *inline_pos) {
@@ -1593,14 +1604,37 @@ extern "C" int32_t pic_prefill_plan_splits(const pic_geom_t *geom, int32_t batch
   // empty CTA, the merge launch and the 4 d + 16 bytes written and read per
   // partial row at 6.5 TB/s
   constexpr double kCtaFixed = 4.0, kCtaEmpty = 0.7, kMerge = 2.0, kTileBytes = 8.5e6;
+  constexpr double kWorthMore = 0.96;  // cost of a count beyond the library's own, against the best
   const double kRowBytes = 4.0 * geom->head_dim + 16.0;
   constexpr int kSms = 152;
   double best = 1e300;
   int best_s = fallback;
   std::vector<double> sm(kSms);
+  auto deal = [&](size_t units, double cost) {  // to the unit that is free first
+    std::pop_heap(sm.begin(), sm.begin() + units, std::greater<double>());
+    sm[units - 1] += cost;
+    std::push_heap(sm.begin(), sm.begin() + units, std::greater<double>());
+  };
+  auto merge_cost = [&](int sp) {
+    return sp == 1 ? 0.0 : kMerge + (double)batch * Hkv * m_tiles * BM * sp * kRowBytes / kTileBytes;
+  };
+  auto clusters_cost = [&](int sp) {  // rotate-on-load: clusters of two pairs on pairs of SMs
+    std::fill(sm.begin(), sm.end(), 0.0);
+    for (int b = 0; b < batch; ++b)
+      for (int hk = 0; hk < Hkv; ++hk)
+        for (int split = 0; split < sp; ++split)
+          for (int pr = 0; pr < npairs; pr += 2) {
+            const int na = pair_tiles[(size_t)b * npairs + pr];
+            const int per = (na + sp - 1) / sp;
+            const int n = std::max(0, std::min(per, na - split * per));
+            deal(kSms / 2, n > 0 ? n + kCtaFixed : kCtaEmpty);
+          }
+    return *std::max_element(sm.begin(), sm.begin() + kSms / 2) + merge_cost(sp);
+  };
+  const double clusters_fallback = clusters_cost(fallback);
   const int max_s = std::min(kMaxSplits, std::max(1, kv_tiles));
   for (int sp = 1; sp <= max_s; ++sp) {
-    const double merge = kMerge + (double)batch * Hkv * m_tiles * BM * sp * kRowBytes / kTileBytes;
+    const double merge = merge_cost(sp);
     // no larger count can win once even a perfect balance costs more than the
     // best: key tiles and fixed costs (of the splits that have keys) over the SMs
     double work = 0.0;
@@ -1610,6 +1644,7 @@ extern "C" int32_t pic_prefill_plan_splits(const pic_geom_t *geom, int32_t batch
         work += na + kCtaFixed * ((na + per - 1) / per);
       }
     if (sp > 1 && work * Hkv / kSms + merge > best) break;
+    if (sp > fallback && clusters_cost(sp) > clusters_fallback) continue;
     std::fill(sm.begin(), sm.end(), 0.0);
     std::make_heap(sm.begin(), sm.end(), std::greater<double>());
     int cuts[4] = {0, 0, 0, npairs};  // groups of pairs in launch order
@@ -1622,12 +1657,10 @@ extern "C" int32_t pic_prefill_plan_splits(const pic_geom_t *geom, int32_t batch
               const int na = pair_tiles[(size_t)b * npairs + pr];
               const int per = (na + sp - 1) / sp;
               const int n = std::max(0, std::min(per, na - split * per));
-              std::pop_heap(sm.begin(), sm.end(), std::greater<double>());
-              sm.back() += n > 0 ? n + kCtaFixed : kCtaEmpty;
-              std::push_heap(sm.begin(), sm.end(), std::greater<double>());
+              deal(kSms, n > 0 ? n + kCtaFixed : kCtaEmpty);
             }
-    const double cost = *std::max_element(sm.begin(), sm.end()) + (sp > 1 ? merge : 0.0);
-    if (cost < best - 1e-9) {
+    const double cost = *std::max_element(sm.begin(), sm.end()) + merge;
+    if (cost < (sp > fallback ? kWorthMore * best : best - 1e-9)) {
       best = cost;
       best_s = sp;
     }

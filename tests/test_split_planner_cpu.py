@@ -57,3 +57,20 @@ def test_decode_split_count_fills_the_gpu():
                 pages = -(-ctx // 16)
                 want = min(-(-8 * 152 // (batch * hkv)), max(1, pages // 16), 64, pages)
                 assert pic.pic_decode_num_splits(g, batch, ctx, 0) == want, (hkv, batch, ctx)
+
+
+@pytest.mark.parametrize("heads,batch,ctx,query", [((32, 8, 128), 4, 1024, 16), ((28, 4, 128), 8, 1024, 1),
+                                                   ((16, 2, 64), 16, 1024, 1), ((28, 4, 128), 4, 4096, 1),
+                                                   ((8, 2, 128), 16, 1024, 16), ((16, 2, 64), 1, 1024, 512)])
+def test_planner_keeps_rotate_on_load_in_one_wave(heads, batch, ctx, query):
+    """Counts beyond the library's own suit the materialised grid, whose short
+    pairs are cheap, but not rotate-on-load's clusters of two pairs, which then
+    take a second wave; the one count both calls use stays at or below it."""
+    hq, hkv, d = heads
+    g = pic.Geometry(1, hq, hkv, d, 5e5)
+    T = 56 + query
+    lens = torch.full((batch,), T, dtype=torch.int32)
+    row = list(range(56)) + list(range(56 + ctx, 56 + ctx + query))
+    pos = torch.tensor([row] * batch, dtype=torch.int32)
+    own = pic.pic_prefill_num_splits(g, batch, T, ctx + T, 0)
+    assert 1 <= pic.pic_prefill_plan_splits(g, ctx + T, lens, pos) <= own
