@@ -77,6 +77,9 @@ pic_status_t encode_tmap_3d(CUtensorMap *map, const void *base, uint64_t inner, 
 // stride (the SW128 operand stride) and the two panels 1024 bytes apart.
 pic_status_t encode_tmap_pages128(CUtensorMap *map, const void *base, uint64_t n_page_heads);
 
+// Document tokens that `batch` requests of up to max_docs documents list: an
+// estimate at the pool's mean length, at most max_ctx per request.
+double listed_tokens(int batch, int max_docs, int n_pool_docs, int64_t pool_tokens, double max_ctx);
 // The relocation of pic_link's documents as a launch of its own, after the
 // layout is on the device (relocate_docs_kernel: a shared document is read
 // once, loads by bulk copies), and whether that pays for a relocation that

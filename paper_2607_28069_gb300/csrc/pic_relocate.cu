@@ -53,7 +53,7 @@ struct RelocArgs {
   const int64_t *doc_start;
   const int32_t *doc_len, *doc_base, *ids, *num_docs, *target, *block_table;
   const int32_t *prefix, *query;  // the link step's (kMapped)
-  bool share;                     // look for documents listed more than once
+  int share;  // occurrences of a document moved together, at most; 1: each by itself, no search
 };
 
 // Moves the positions a CTA of relocate_kernel set up (s_src / s_dst / s_doc,
@@ -131,10 +131,10 @@ __global__ void __launch_bounds__(kThreads) relocate_kernel(RelocArgs a, RopePar
 // The per-document form, by pool document: a document that several listed
 // occurrences share (requests of a batch that retrieved the same document, a
 // boundary block repeated in one request) is read once and written to all of
-// them.  CTA (slice, k, b) first finds the other occurrences of its document
-// among the batch's document lists -- up to kMaxShare of them form a group --
-// and then moves every r-th chunk of kTok tokens from its own rank on (r: the
-// group's size; of those, every gridDim.x-th from its slice on) to all r
+// them.  CTA (k, b, slice) first finds the other occurrences of its document
+// among the batch's document lists -- up to a.share of them, at most kMaxShare,
+// form a group (share_limit) -- and then moves every r-th chunk of kTok tokens from its own rank on (r: the
+// group's size; of those, every gridDim.z-th from its slice on) to all r
 // places: token j of the document (pool row doc_start + j, compiled at base +
 // j) goes to logical position target + j of each occurrence, rotated by its
 // delta = target - base.  HBM-bound: 1 + r row transfers a token instead of 2r.
@@ -142,7 +142,8 @@ __global__ void __launch_bounds__(kThreads) relocate_kernel(RelocArgs a, RopePar
 // The work of a CTA is a list of units (chunk, layer, block of kv heads) of at
 // most 16 KB of K and 16 KB of V, contiguous in the pool: bulk copies bring
 // them into a ring of two stages while the unit before is rotated and stored,
-// so loads stay in flight whatever r is.  Three CTAs an SM.  Measured against
+// so loads stay in flight whatever r is.  Three CTAs an SM (two with per-layer
+// tables in chunks of 32 tokens at d = 128, for their shared memory).  Measured against
 // a CTA that held 16 tokens in registers and knew one occurrence (four layers
 // unless stated): 8 requests with 16 of 64 1024-token documents 720 -> 510 us
 // (6.3 TB/s of the bytes that must move), 16 with 32 of 64 on 4 kv heads and
@@ -164,7 +165,8 @@ template <int D, int kTok, bool kLayerRope, bool kMapped>
 __global__ void __launch_bounds__(kThreads, 3) relocate_docs_kernel(RelocArgs a, RopeParams rp) {
   pdl_entry();
   constexpr int HALF = D / 2, KC = D / 16, VC = D / 8;
-  const int k = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, lane = tid & 31, style = rp.style;
+  const int k = blockIdx.x, b = blockIdx.y, slice = blockIdx.z;
+  const int tid = threadIdx.x, lane = tid & 31, style = rp.style;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t ring = (smem_u32(smem_raw) + 127u) & ~127u;
   __shared__ uint32_t s_mask[kMaxScan / 32];  // listed documents equal to this one
@@ -181,8 +183,8 @@ __global__ void __launch_bounds__(kThreads, 3) relocate_docs_kernel(RelocArgs a,
 
   // ---- this occurrence, and the first 256 listed documents beside it: all
   // loads independent of one another
-  const int listed = (int)gridDim.z * a.max_docs, own = b * a.max_docs + k;
-  const bool scan = a.share && listed <= kMaxScan;
+  const int listed = (int)gridDim.y * a.max_docs, own = b * a.max_docs + k;
+  const bool scan = a.share > 1 && listed <= kMaxScan;
   auto target_ok = [&](long long t, int len) {
     return t >= 0 && (kMapped || t + len <= (long long)a.max_pages * 16);
   };
@@ -201,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 3) relocate_docs_kernel(RelocArgs a,
   };
   Entry e0{-1, -1};
   if (scan) e0 = entry(tid);
-  const bool report = !kMapped && tid == 0 && blockIdx.x == 0;
+  const bool report = !kMapped && tid == 0 && slice == 0;
   const int m = a.num_docs[b];
   if (m < 0 || m > a.max_docs) {
     if (report && k == 0) dev_fail(a.status, PIC_DEV_BAD_REQUEST, b);
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(kThreads, 3) relocate_docs_kernel(RelocArgs a,
     if (report) dev_fail(a.status, target < 0 ? PIC_DEV_BAD_POSITION : PIC_DEV_BLOCK_TABLE_SHORT, b);
     return;
   }
-  if (!kMapped && blockIdx.x == 0 && tid < 32) {  // targets of two listed documents must not overlap
+  if (!kMapped && slice == 0 && tid < 32) {  // targets of two listed documents must not overlap
     bool clash = false;
     for (int k2 = tid; k2 < m; k2 += 32) {
       if (k2 == k) continue;
@@ -241,6 +243,7 @@ __global__ void __launch_bounds__(kThreads, 3) relocate_docs_kernel(RelocArgs a,
   // ---- the group: the valid occurrences of the document, in list order
   int cnt = 1, rank = 0;
   if (scan) {
+    if (slice >= (n + kTok - 1) / kTok) return;  // no chunk for this slice, whatever the group
     const int words = (listed + 31) / 32;
     for (int e = tid; e < words * 32; e += kThreads) {
       const Entry x = e == tid ? e0 : entry(e);
@@ -266,15 +269,15 @@ __global__ void __launch_bounds__(kThreads, 3) relocate_docs_kernel(RelocArgs a,
       return base_w + __popc(s_mask[w] & ((1u << (e & 31)) - 1u));
     };
     rank = rank_of(own);
-    const int first = rank / kMaxShare * kMaxShare;  // the group's first rank
+    const int first = rank / a.share * a.share;  // the group's first rank
     for (int e = tid; e < words * 32; e += kThreads) {
       const int r = rank_of(e) - first;
-      if ((s_mask[e / 32] >> lane & 1u) && r >= 0 && r < kMaxShare) {
+      if ((s_mask[e / 32] >> lane & 1u) && r >= 0 && r < a.share) {
         s_tb[r] = e / a.max_docs;
         s_tt[r] = e == tid ? e0.target : a.target[e];
       }
     }
-    cnt = min(total - first, kMaxShare);
+    cnt = min(total - first, a.share);
     rank -= first;
   } else if (tid == 0) {
     s_tb[0] = b;
@@ -288,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, 3) relocate_docs_kernel(RelocArgs a,
   if (lo >= hi) return;
   const int j_lo = (int)lo, n_tok = (int)(hi - lo);
   const int chunks = (n_tok + kTok - 1) / kTok;
-  const int c_first = rank + cnt * (int)blockIdx.x, c_step = cnt * (int)gridDim.x;
+  const int c_first = rank + cnt * slice, c_step = cnt * (int)gridDim.z;
   if (c_first >= chunks) return;
   const int my_chunks = (chunks - c_first + c_step - 1) / c_step;
   const int hkv = a.hkv, hb = min(hkv, kUnit / (kTok * D)), hblocks = (hkv + hb - 1) / hb;
@@ -517,17 +520,37 @@ __device__ __forceinline__ void move_positions(const RelocArgs &a, const RopePar
   }
 }
 
-// Bytes a relocation moves (host estimate: the listed documents at the pool's
-// mean length) from which the search for shared documents pays for itself:
-// it costs a CTA about a microsecond before its first copy (2 requests of 8
-// documents of 512 tokens, 67 MB: 24 us with the search, 19 without; 8 of 16
-// documents of 290, 150 MB: 69 us before, 49 with it).
+// Tokens of a chunk, by the elements of a token's K row (units of at most 16 KB).
+constexpr int chunk_tokens(int row) { return row >= 1024 ? 8 : row >= 512 ? 16 : 32; }
+
+// Occurrences of a document that are moved together, at most (1: no search), for
+// a relocation of `tokens` listed document tokens (host estimate: the pool's mean
+// length) that moves `bytes`.  The search costs a CTA about a microsecond before
+// its first copy, which pays from kShareBytes on (2 requests of 8 documents of
+// 512 tokens, 67 MB: 24 us with it, 19 without).  And a chunk that r occurrences
+// share is one CTA's work instead of r CTAs', so groups stay small enough that
+// two waves of chunks are left if every document has r occurrences: with groups
+// of up to 8 in any case, 16 requests listing the same two documents of 64 tokens,
+// 16 layers, took 4.4 times as long as without sharing, and 84 of 153 shapes with
+// shared documents from 128 MB on got slower by it (1.21 times as long on average);
+// with this limit five, by up to 16% (640 listed documents of 100 tokens), and 0.94
+// on average (8 requests with 16 documents of 1024 tokens, one layer 147 -> 108 us).
 constexpr double kShareBytes = 128e6;
+constexpr int kWave = 3 * 152;  // CTAs resident at once
+inline int share_limit(double tokens, int row, double bytes) {
+  if (bytes < kShareBytes) return 1;
+  return (int)std::max(1.0, std::min<double>(kMaxShare, tokens / chunk_tokens(row) / (2 * kWave)));
+}
 
 // Launch of the per-document form.  Slices per listed document: each CTA
 // walks every slices-th chunk of its share of the document; few documents get
 // more slices (up to one chunk per CTA), so that a small request still fills
-// the GPU (CTAs past a document's last chunk exit).
+// the GPU, but no more than a document of twice the pool's mean length has
+// chunks.  The slices come last in the launch order: CTAs past a document's
+// last chunk exit, and among working ones they left the SMs unevenly filled (one
+// request of 8 documents of 512 tokens, 16/2 heads of 64, 16 layers: 47% of the SM
+// cycles active, 37 us; in this order 30; 720 relocations 0.70 of the time before
+// the bulk copies on average, 0.78 with the slices first).
 template <int D, int kTok, bool kMapped>
 cudaError_t launch_docs_as(const RelocArgs &a, const RopeParams &rp, const dim3 &grid,
                            cudaStream_t stream) {
@@ -543,15 +566,19 @@ cudaError_t launch_docs(const pic_geom_t *geom, const RelocArgs &a, const RopePa
                         cudaStream_t stream) {
   const int row = geom->num_kv_heads * geom->head_dim;
   const long long docs_total = (long long)batch * a.max_docs;
-  const int slices = (int)std::min<long long>(128, std::max<long long>(16, (8 * 152 + docs_total - 1) / docs_total));
-  const dim3 grid(slices, a.max_docs, batch);
+  const int tok = chunk_tokens(row);
+  const double mean_chunks = (double)a.pool_tokens / std::max(a.n_pool_docs, 1) / tok;
+  const long long most = std::max(1ll, (long long)std::ceil(2.0 * std::min(mean_chunks, 1e6)));
+  const long long want = std::max<long long>(16, (8 * 152 + docs_total - 1) / docs_total);
+  const int slices = (int)std::min({128ll, want, most});
+  const dim3 grid(a.max_docs, batch, slices);
   if (geom->head_dim == 128)
-    return row >= 1024 ? launch_docs_as<128, 8, kMapped>(a, rp, grid, stream)
-           : row >= 512 ? launch_docs_as<128, 16, kMapped>(a, rp, grid, stream)
-                        : launch_docs_as<128, 32, kMapped>(a, rp, grid, stream);
-  return row >= 1024 ? launch_docs_as<64, 8, kMapped>(a, rp, grid, stream)
-         : row >= 512 ? launch_docs_as<64, 16, kMapped>(a, rp, grid, stream)
-                      : launch_docs_as<64, 32, kMapped>(a, rp, grid, stream);
+    return tok == 8    ? launch_docs_as<128, 8, kMapped>(a, rp, grid, stream)
+           : tok == 16 ? launch_docs_as<128, 16, kMapped>(a, rp, grid, stream)
+                       : launch_docs_as<128, 32, kMapped>(a, rp, grid, stream);
+  return tok == 8    ? launch_docs_as<64, 8, kMapped>(a, rp, grid, stream)
+         : tok == 16 ? launch_docs_as<64, 16, kMapped>(a, rp, grid, stream)
+                     : launch_docs_as<64, 32, kMapped>(a, rp, grid, stream);
 }
 
 }  // namespace
@@ -589,11 +616,17 @@ cudaError_t launch_link_relocation(const pic_geom_t *geom, const RopeParams &rp,
   a.target = doc_offset;
   a.prefix = prefix_len;
   a.query = query_len;
-  a.share = true;
+  const double tokens = listed_tokens(batch, max_docs, n_pool_docs, pool_tokens, max_ctx);
+  const int row = geom->num_kv_heads * geom->head_dim;
+  a.share = share_limit(tokens, row, 8.0 * tokens * row * (layer_end - layer_begin));
   return launch_docs<true>(geom, a, rp, batch, stream);
 }
 
 bool link_relocation_apart(double bytes) { return bytes >= kShareBytes; }
+
+double listed_tokens(int batch, int max_docs, int n_pool_docs, int64_t pool_tokens, double max_ctx) {
+  return batch * std::min((double)max_docs * pool_tokens / std::max(n_pool_docs, 1), max_ctx);
+}
 }  // namespace pic
 
 extern "C" pic_status_t pic_relocate_mapped(const pic_geom_t *geom, int32_t batch,
@@ -718,8 +751,9 @@ extern "C" pic_status_t pic_relocate(const pic_geom_t *geom, int32_t batch, int3
   a.num_docs = req_num_docs;
   a.target = doc_target;
   a.block_table = block_table;
-  a.share = 8.0 * batch * max_docs * ((double)pool_tokens / n_pool_docs) * geom->num_kv_heads *
-                geom->head_dim * (layer_end - layer_begin) >= kShareBytes;
+  const double tokens = listed_tokens(batch, max_docs, n_pool_docs, pool_tokens, 16.0 * max_pages);
+  const int row = geom->num_kv_heads * geom->head_dim;
+  a.share = share_limit(tokens, row, 8.0 * tokens * row * (layer_end - layer_begin));
   cudaError_t e = launch_docs<false>(geom, a, rp, batch, stream);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "pic_relocate launch");

@@ -1,11 +1,12 @@
 """Documents that several listed occurrences share: pic_relocate reads each once
-and writes it to every occurrence (relocate_docs_kernel), from 128 MB of
-relocation on, and pic_link uses the same kernel.  Both are compared bit for
-bit with pic_relocate_mapped, which moves position by position and knows no
-sharing: groups of one to more than kMaxShare = 8 occurrences, a document
-repeated in one request, head counts that leave a remainder block of heads,
-chunks of 8, 16 and 32 tokens with remainders, both RoPE styles, per-layer
-rotary tables, document lists beyond the 2048 a CTA searches."""
+and writes it to every occurrence (relocate_docs_kernel), in large relocations
+with enough document tokens for groups of two or more, and large pic_links use
+the same kernel.  Both are compared bit for bit with pic_relocate_mapped, which
+moves position by position and knows no sharing: groups of two to kMaxShare = 8
+occurrences, more occurrences than a group takes, a document repeated in one
+request, head counts that leave a remainder block of heads, chunks of 8, 16 and
+32 tokens with remainders, both RoPE styles, per-layer rotary tables, document
+lists beyond the 2048 a CTA searches, and relocations too small to search."""
 import pytest
 import torch
 
@@ -19,33 +20,39 @@ def _spec(name, **kw):
 
 
 CASES = {
-    # name: (spec, rope style, per-layer tables)
-    "pairs": (_spec("pairs", layers=4, q_heads=32, kv_heads=8, head_dim=128, batch=3, pool_docs=9,
-                    docs_per_request=6, doc_len=(100, 700)), 0, False),
+    # name: (spec, rope style, per-layer tables, group size)
+    "pairs": (_spec("pairs", layers=2, q_heads=32, kv_heads=8, head_dim=128, batch=3, pool_docs=9,
+                    docs_per_request=6, doc_len=(900, 2100)), 0, False, 3),
     "groups_over_8": (_spec("groups_over_8", layers=2, q_heads=32, kv_heads=8, head_dim=128,
-                            batch=19, pool_docs=3, docs_per_request=3, doc_len=(1, 333),
-                            span_len=(0, 5)), 1, False),
-    "repeated": (_spec("repeated", layers=5, q_heads=8, kv_heads=4, head_dim=128, batch=2,
-                       pool_docs=4, docs_per_request=7, doc_len=(300, 1700),
-                       fixed_order=(0, 2, 1, 0, 3, 1, 0)), 0, True),
+                            batch=19, pool_docs=3, docs_per_request=3, doc_len=(1001, 1333),
+                            span_len=(0, 5)), 1, False, 8),
+    "repeated": (_spec("repeated", layers=2, q_heads=8, kv_heads=4, head_dim=128, batch=2,
+                       pool_docs=4, docs_per_request=7, doc_len=(2900, 5100),
+                       fixed_order=(0, 2, 1, 0, 3, 1, 0)), 0, True, 4),
     "heads_12": (_spec("heads_12", layers=2, q_heads=24, kv_heads=12, head_dim=128, batch=4,
-                       pool_docs=5, docs_per_request=4, doc_len=(200, 900)), 1, False),
-    "d64_h3": (_spec("d64_h3", layers=6, q_heads=6, kv_heads=3, head_dim=64, batch=5, pool_docs=6,
-                     docs_per_request=5, doc_len=(500, 1500)), 0, False),
+                       pool_docs=5, docs_per_request=4, doc_len=(1500, 2400)), 1, False, 4),
+    "d64_h3": (_spec("d64_h3", layers=2, q_heads=6, kv_heads=3, head_dim=64, batch=5, pool_docs=6,
+                     docs_per_request=5, doc_len=(5000, 7000)), 0, False, 5),
     "d64_h16_tables": (_spec("d64_h16_tables", layers=3, q_heads=16, kv_heads=16, head_dim=64,
-                             batch=4, pool_docs=5, docs_per_request=5, doc_len=(150, 800)), 0, True),
+                             batch=4, pool_docs=5, docs_per_request=5, doc_len=(900, 2200)), 0, True,
+                       4),
     "beyond_scan": (_spec("beyond_scan", layers=2, q_heads=8, kv_heads=4, head_dim=128, batch=17,
-                          pool_docs=130, docs_per_request=128, doc_len=(1, 30)), 0, False),
-    # one request: nothing shared, but large enough for the three-launch link
+                          pool_docs=130, docs_per_request=128, doc_len=(1, 30)), 0, False, 2),
+    # one request: nothing shared, and too few tokens to look for it
     "one_request": (_spec("one_request", layers=10, q_heads=8, kv_heads=2, head_dim=128, batch=1,
-                          pool_docs=20, docs_per_request=12, doc_len=(300, 1000)), 0, False),
+                          pool_docs=20, docs_per_request=12, doc_len=(300, 1000)), 0, False, 1),
 }
 
 
 def _path(name):
     from paper_2607_28069_gb300.pipeline import CacheHitPath
-    spec, style, tables = CASES[name]
+    spec, style, tables, _ = CASES[name]
     wl = generate(spec, device="cuda", gen_device="cuda")
+    # a capacity from which the link is three launches (2200 CTAs of a page or two)
+    wl.max_ctx = max(wl.max_ctx, -(-2200 // spec.batch) * 32)
+    table = torch.full((spec.batch, -(-wl.max_ctx // 16)), -1, dtype=torch.int32, device="cuda")
+    table[:, :wl.block_table.shape[1]] = wl.block_table
+    wl.block_table = table
     freqs = None
     if tables:
         i = torch.arange(spec.head_dim // 2, dtype=torch.float64)
@@ -59,8 +66,13 @@ def test_shared_documents_bit_identical(cuda_lib, name):
     import paper_2607_28069_gb300 as pic
     path = _path(name)
     spec = path.wl.spec
-    assert 8 * spec.batch * path.max_ctx * spec.kv_heads * spec.head_dim * spec.layers >= 128e6 \
-        or name == "beyond_scan"
+    # the group size is what the test says it is
+    row = spec.kv_heads * spec.head_dim
+    tokens = spec.batch * spec.docs_per_request * path.wl.k_pool.shape[1] / spec.pool_docs
+    chunk = 8 if row >= 1024 else 16 if row >= 512 else 32
+    large = 8 * tokens * row * spec.layers >= 128e6
+    group = max(1, min(8, int(tokens / chunk / 912))) if large else 1
+    assert group == CASES[name][3]
     path.compose()
     path.relocate_mapped()
     k_ref, v_ref = path.k_cache.clone(), path.v_cache.clone()
@@ -78,7 +90,9 @@ def test_shared_documents_bit_identical(cuda_lib, name):
     path.k_cache.zero_(), path.v_cache.zero_(), path.ws_prefill.zero_()
     for m in maps:
         getattr(path, m).fill_(-7)
+    before = pic.pic_launch_count()
     path.link(0)
+    assert pic.pic_launch_count() - before == 3
     assert torch.equal(path.k_cache, k_ref) and torch.equal(path.v_cache, v_ref)
     assert torch.equal(path.ws_prefill[:packed], ws_ref)
     for m in maps:
