@@ -271,8 +271,8 @@ pic_status_t pic_relocate_mapped(const pic_geom_t *geom, int32_t batch, int32_t 
 /*
  * pic_link -- pic_compose, pic_relocate_mapped (layers [layer_begin, layer_end)) and
  * pic_append_inline (layer append_layer, or none when append_layer < 0) in one
- * call, a single launch unless the relocation is large: the link step of a cache hit (Eqs. 1-3; appendix
- * "Position-Independent Linking").  Every argument means what it means for
+ * call, a single launch unless the link is large: the link step of a cache hit
+ * (Eqs. 1-3; appendix "Position-Independent Linking").  Every argument means what it means for
  * those three calls, and every output -- the layout (doc_offset, doc_delta,
  * slot_mapping, tok_map, inline_pos, ctx_len), the stitched K/V of the
  * documents and of the appended inline tokens, and the packed queries at the
@@ -282,9 +282,13 @@ pic_status_t pic_relocate_mapped(const pic_geom_t *geom, int32_t batch, int32_t 
  * every layer in turn, plus one inline token slot, and derives the layout it
  * needs itself, so the three dependent chains of memory round trips become
  * one.  Requests with more than 256 documents (max_docs > 256) run the three
- * calls in order instead, and a relocation of 128 MB or more three launches in
- * that order, of which the second reads a document that several requests (or
- * one request several times) list only once.
+ * calls in order instead.  Links with much to move (600 MB of K and V read and
+ * written, estimated from max_docs documents per request at the pool's mean
+ * length) or with a large batch * max_ctx (2200 and more CTAs) are three
+ * launches in that order, of which the second moves up to 8 occurrences of a
+ * document that several requests (or one request several times) list with one
+ * read (batches of up to 2048 listed documents; fewer occurrences at a time
+ * where the listed tokens are few).
  * workspace: the prefill workspace of pic_append_inline (only its leading
  *   packed-query part is written); may be NULL when append_layer < 0.
  * One launch (or three), asynchronous on `stream`;

@@ -284,7 +284,7 @@ def pic_link(geom: Geometry, doc_len, doc_base_pos, doc_token_start, req_doc_ids
              inline_len, k_cache, v_cache, doc_offset, doc_delta, slot_mapping, tok_map, inline_pos,
              ctx_len, workspace, stream=None, span_len=None):
     """pic_compose + pic_relocate + pic_append_inline (append_layer, or none if < 0)
-    in one launch; q/k_new/v_new are the append layer's inline projections;
+    in one call (one launch, three for large batches); q/k_new/v_new are the append layer's inline projections;
     span_len as for pic_compose."""
     st = (_nat or _native()).link(
         geom, doc_len, doc_base_pos, doc_token_start, req_doc_ids, req_num_docs, span_len,

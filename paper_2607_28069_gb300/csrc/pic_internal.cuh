@@ -82,9 +82,10 @@ pic_status_t encode_tmap_pages128(CUtensorMap *map, const void *base, uint64_t n
 double listed_tokens(int batch, int max_docs, int n_pool_docs, int64_t pool_tokens, double max_ctx);
 // The relocation of pic_link's documents as a launch of its own, after the
 // layout is on the device (relocate_docs_kernel: a shared document is read
-// once, loads by bulk copies), and whether that pays for a relocation that
-// moves up to `bytes`.
-bool link_relocation_apart(double bytes);
+// once, loads by bulk copies), and whether that pays for a relocation of about
+// `tokens` document tokens (of `row` K elements each) in `layers` layers, against
+// one launch of `ctas` CTAs.
+bool link_relocation_apart(double tokens, int row, int layers, long long ctas);
 cudaError_t launch_link_relocation(const pic_geom_t *geom, const RopeParams &rp, int batch,
                                    int max_docs, int n_pool_docs, const void *k_pool,
                                    const void *v_pool, int64_t pool_tokens,

@@ -579,14 +579,18 @@ extern "C" pic_status_t pic_link(
   int32_t *status = device_status_ptr();
   if (!status) return fail(PIC_ERR_CUDA, "pic_link: no device status word");
 
+  // one page per CTA when a token carries >= 1024 K elements, else two
+  const bool wide = geom->num_kv_heads * geom->head_dim >= 1024;
+  const int tok = wide ? 16 : 32;
+  const int n_pages = (max_ctx + tok - 1) / tok, t_slots = std::max(max_inline, (R_pad + G - 1) / G);
+  const int ctas_x = do_append ? std::max(n_pages, t_slots) : n_pages;
+
   // From some size on the layout, the relocation (which reads a document that
   // requests share once and loads by bulk copies) and the append are launches
-  // of their own: four layers of 8 requests with 16 of 64 1024-token documents
-  // 740 -> 533 us, no document shared (16 x 350 tokens) 280 -> 251, one layer
-  // of 16 x 290 tokens 87 -> 70.  Below, one launch saves two and their
-  // dependencies (8 x 512 tokens: 14 us against about 20).
-  if (link_relocation_apart(8.0 * batch * max_ctx * geom->num_kv_heads * geom->head_dim *
-                            (layer_end - layer_begin))) {
+  // of their own (see link_relocation_apart).
+  if (link_relocation_apart(listed_tokens(batch, max_docs, n_pool_docs, pool_tokens, max_ctx),
+                            geom->num_kv_heads * geom->head_dim, layer_end - layer_begin,
+                            (long long)n_pages * batch)) {
     const int32_t *tin = do_append ? inline_len : nullptr;
     st = compose_layout(geom, batch, max_docs, n_pool_docs, doc_len, doc_base_pos, doc_token_start,
                         req_doc_ids, req_num_docs, span_len, prefix_len, query_len, block_table,
@@ -619,11 +623,8 @@ extern "C" pic_status_t pic_link(
   a.hkv = geom->num_kv_heads;
   a.G = G;
   a.R_pad = R_pad;
-  a.t_slots = std::max(max_inline, (R_pad + G - 1) / G);
-  // one page per CTA when a token carries >= 1024 K elements, else two
-  const bool wide = geom->num_kv_heads * geom->head_dim >= 1024;
-  const int tok = wide ? 16 : 32;
-  a.n_pages = (max_ctx + tok - 1) / tok;
+  a.t_slots = t_slots;
+  a.n_pages = n_pages;
   a.num_pages = num_pages;
   a.pool_tokens = pool_tokens;
   a.doc_len = doc_len;
@@ -652,7 +653,7 @@ extern "C" pic_status_t pic_link(
   a.qpack = static_cast<__nv_bfloat16 *>(workspace);
   a.status = status;
 
-  dim3 grid((unsigned)(do_append ? std::max(a.n_pages, a.t_slots) : a.n_pages), batch);
+  dim3 grid((unsigned)ctas_x, batch);
   const dim3 block(kThreads);
   cudaError_t e;
   const bool per_layer = rp.layer_theta != nullptr;

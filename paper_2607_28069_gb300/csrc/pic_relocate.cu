@@ -622,7 +622,19 @@ cudaError_t launch_link_relocation(const pic_geom_t *geom, const RopeParams &rp,
   return launch_docs<true>(geom, a, rp, batch, stream);
 }
 
-bool link_relocation_apart(double bytes) { return bytes >= kShareBytes; }
+// One launch derives the layout in every CTA, empty ones included, and reads a
+// shared document once per occurrence; three launches cost about 10 us of
+// launches and dependencies.  Measured over 1140 shapes of 1 to 16 requests (1,
+// 4, 16 layers; capacity max_ctx one and four times the context): from 600 MB in
+// two waves of chunks, or from 2200 CTAs on, the three launches are faster (8 requests with 16 of 64 documents
+// of 1024 tokens, four layers 740 -> 533 us; 4 with 16 of 1024 tokens, one layer
+// 131 -> 89; one of 8 documents of 512 tokens, capacity 131k, one layer 60 -> 22),
+// but for three shapes, by 7 to 16%.  Below, one launch is (one request of 8
+// documents of 512 tokens, one layer, capacity 16k: 14.4 us against 21.6).  A line
+// at 128 MB of capacity made 105 of them up to 52% slower than one launch.
+bool link_relocation_apart(double tokens, int row, int layers, long long ctas) {
+  return (8.0 * tokens * row * layers >= 600e6 && tokens / chunk_tokens(row) >= 2 * kWave) || ctas >= 2200;
+}
 
 double listed_tokens(int batch, int max_docs, int n_pool_docs, int64_t pool_tokens, double max_ctx) {
   return batch * std::min((double)max_docs * pool_tokens / std::max(n_pool_docs, 1), max_ctx);

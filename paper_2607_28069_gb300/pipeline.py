@@ -249,7 +249,7 @@ class CacheHitPath:
                             self.slot_mapping, wl.num_pages, self.k_cache, self.v_cache,
                             layer_begin, layer_end)
 
-    # -- a1 + a2 + a3 + a4 (first layer) in one launch
+    # -- a1 + a2 + a3 + a4 (first layer) in one call
     def link(self, append_layer: int = 0):
         wl = self.wl
         L = wl.spec.layers
@@ -326,7 +326,7 @@ class CacheHitPath:
         """The cache-hit path up to the first token: layout, re-rotation and
         stitching of every layer, then every layer's inline prefill.  With
         ``linked`` the layout, the relocation and the first layer's inline
-        append are one pic_link launch; otherwise the separate calls."""
+        append are one pic_link call; otherwise the separate calls."""
         if linked:
             self.link(0)
             self.attend(0)

@@ -164,3 +164,30 @@ def test_large_links_back_to_back(cuda_lib):
         for got, want in zip(zip(kc, vc, ws), ref):
             assert all(torch.equal(a, b) for a, b in zip(got, want))
     assert pic.pic_device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("docs,capacity,launches", [((4, 300), 1, 1), ((4, 300), 8, 1),
+                                                    ((4, 300), 32, 3), ((40, 1000), 1, 3)])
+def test_link_form_follows_the_documents(cuda_lib, docs, capacity, launches):
+    """The link of a short request stays one launch where the capacity max_ctx is
+    several times its context; many CTAs or much to move make it three.  Both
+    forms give the three separate calls' caches and layout, bit for bit."""
+    import paper_2607_28069_gb300 as pic
+    from paper_2607_28069_gb300.pipeline import CacheHitPath
+    spec = _spec("form", layers=2, q_heads=32, kv_heads=8, head_dim=128, batch=2, pool_docs=docs[0],
+                 docs_per_request=docs[0], doc_len=(docs[1], docs[1]))
+    wl = generate(spec, device="cuda", gen_device="cuda")
+    table = torch.full((2, wl.block_table.shape[1] * capacity), -1, dtype=torch.int32, device="cuda")
+    table[:, :wl.block_table.shape[1]] = wl.block_table
+    wl.block_table, wl.max_ctx = table, wl.max_ctx * capacity
+    path = CacheHitPath(wl)
+    path.compose(), path.relocate_mapped(), path.append(0)
+    maps = ("doc_offset", "doc_delta", "slot_mapping", "tok_map", "inline_pos", "ctx_len")
+    ref = [path.k_cache.clone(), path.v_cache.clone()] + [getattr(path, m).clone() for m in maps]
+    path.k_cache.zero_(), path.v_cache.zero_()
+    before = pic.pic_launch_count()
+    path.link(0)
+    assert pic.pic_launch_count() - before == launches
+    got = [path.k_cache, path.v_cache] + [getattr(path, m) for m in maps]
+    assert all(torch.equal(a, b) for a, b in zip(got, ref))
+    assert pic.pic_device_status() == (0, 0)
