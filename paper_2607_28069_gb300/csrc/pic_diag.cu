@@ -129,10 +129,10 @@ __device__ uint32_t four_regions(const int32_t *s_off, const int32_t *s_bnd, int
 // The two exponentials a term take MUFU 1024 cycles a tile and the MMAs as
 // long; a tile takes about 2350, in the compute warps' dependent chains (two
 // warps an SMSP, in step on the same tile).  One layer of two requests of 14k
-// document tokens, 256 query tokens each: 181 us with 32 columns read at a time,
-// scalar scaling and one masked sum per region at every boundary, 174 with the
-// tile in registers and packed pairs, 162 with the split count's cost model
-// fitted to it.
+// document tokens, 256 query tokens each: 181 us with 32 columns read at a time
+// and scalar scaling, 174 with the tile in registers and packed pairs, 162 with
+// the split count's cost model fitted to it, 142 as it is (a third K stage, the
+// boundary chunks on packed terms too).
 template <int D, int NS>
 __global__ void __launch_bounds__(kThreads, 1)
     deviation_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_ka,
@@ -327,10 +327,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       // two chunks of 32.  The terms of a chunk are computed without branches
       // (the exponentials pipeline); a chunk whose keys all lie in one region
       // (the region bytes are the same for every row) is summed at once, one in
-      // no region is skipped, one across a single region or document boundary
-      // takes two sums, and only a chunk with more boundaries is summed region
-      // by region.  A key after a row's position (an inline span taken as a
-      // query row before a later document) has p_A = p_B = 0.
+      // no region is skipped, and one across a region or document boundary is
+      // summed region by region.  A key after a row's position (an inline span
+      // taken as a query row before a later document) has p_A = p_B = 0.
       const int wq = warp & 3, half = (warp - 2) >> 2;
       const int row = wq * 32 + lane, rg = r0 + row;
       float la = INFINITY, lb = INFINITY;  // rows past the query rows add nothing
@@ -411,34 +410,21 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (c > lim) d[c] = 0.f;
             if (c + 1 > lim) d[c + 1] = 0.f;
           }
-          // one boundary: keys below n_lo in reg0, the rest in reg1
-          const int reg1 = __shfl_sync(0xffffffffu, rb[h], 31);
-          const uint32_t rest = __ballot_sync(0xffffffffu, rb[h] == reg1);
-          if ((same & (same + 1)) == 0 && (rest | same) == 0xffffffffu) {
-            const int n_lo = same == 0xffffffffu ? 32 : __popc(same);
-            float lo0 = 0.f, lo1 = 0.f, hi0 = 0.f, hi1 = 0.f;
+          // one masked sum per region that the chunk touches; a second form of it for
+          // a single boundary (two sums by position) enlarged the unrolled loop: 6
+          // requests of 60 documents of 200 tokens, 5 query tokens 75.9 us with it,
+          // 65.9 without; 2 requests of 14k document tokens 143.5 and 142.2
+#pragma unroll 1
+          for (int i = 0; i < a.n_regions; ++i) {
+            const uint32_t in = __ballot_sync(0xffffffffu, rb[h] == i);
+            if (!in) continue;
+            float v0 = 0.f, v1 = 0.f;
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
-              lo0 += c < n_lo ? d[c] : 0.f;
-              hi0 += c < n_lo ? 0.f : d[c];
-              lo1 += c + 1 < n_lo ? d[c + 1] : 0.f;
-              hi1 += c + 1 < n_lo ? 0.f : d[c + 1];
-            }
-            add_to(reg0, lo0 + lo1);
-            add_to(reg1, hi0 + hi1);
-          } else {
-#pragma unroll 1
-            for (int i = 0; i < a.n_regions; ++i) {
-              const uint32_t in = __ballot_sync(0xffffffffu, rb[h] == i);
-              if (!in) continue;
-              float v0 = 0.f, v1 = 0.f;
-#pragma unroll
-              for (int c = 0; c < 32; c += 2) {
-                v0 += (in >> c) & 1u ? d[c] : 0.f;
-                v1 += (in >> (c + 1)) & 1u ? d[c + 1] : 0.f;
-              }
-              add_to(i, v0 + v1);
-            }
+              v0 += (in >> c) & 1u ? d[c] : 0.f;
+              v1 += (in >> (c + 1)) & 1u ? d[c + 1] : 0.f;
+          }
+            add_to(i, v0 + v1);
           }
         }
       }
