@@ -525,7 +525,8 @@ pic_status_t pic_attend_decode(const pic_geom_t *geom, int32_t layer, int32_t ba
  * no counterpart: this is a deployment convenience of this library.
  *
  * Same arguments and results as pic_attend_decode, without the workspace:
- * the scratch (per-split partial softmax states) lives in an
+ * the scratch (per-split partial softmax states, sized as by
+ * pic_decode_workspace_size) lives in an
  * 8 MiB array inside the library that every GPU which loads it holds until
  * the process exits.  The call allocates nothing.
  *  - The first call on a device (with that device current) looks the array

@@ -482,6 +482,8 @@ __global__ void decode_combine_kernel(Params p) {
 
 struct Plan {
   int splits, pages_per_split;
+  // q_bytes: the start of the scratch, once the rotated queries, which stay in
+  // shared memory now; kept so that the sizes callers have laid out still hold
   size_t q_bytes, po_bytes, pml_bytes, total;
 };
 

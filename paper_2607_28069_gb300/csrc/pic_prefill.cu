@@ -14,16 +14,18 @@
 //     g*G + r % G of inline token r / G.  One 128-row tile therefore holds
 //     every query head that shares a K/V tile.
 // pic_attend_prefill (one layer):
-//  1. attn_kernel: one CTA per (128-row query tile, key split, kv head,
-//     request).  Warp-specialised: warp 0 issues TMA loads (Q once, then
-//     128-key K and V tiles page by page from the paged cache through the
-//     block table, 3-stage ring; its 32 lanes issue the 32 page boxes of a
-//     tile at once and fetch the next tile's block-table entries ahead), warp 1 issues tcgen05.mma (S = Q K^T into
-//     TMEM, then O += P V with P read from TMEM), warps 2-5 run the online
-//     softmax on S rows straight from TMEM (one thread per row), write P back
-//     to TMEM as bf16 over S, rescale O only when the running maximum grew by
-//     more than 2^8, and finally normalise O.  Scores are kept in the log2
-//     domain (scale folded with log2 e) and exponentiated with ex2.approx.
+//  1. attn_kernel: one CTA per (pair of 128-row query tiles, key split, kv head,
+//     request).  Warp-specialised: warp 0 issues TMA loads of the queries and of
+//     128-key K tiles (3-stage ring, one box per page from the paged cache
+//     through the block table, the next tile's entries looked up ahead), warp 10
+//     of V tiles (2 stages), warp 1 issues tcgen05.mma (S = Q K^T into TMEM, then
+//     O += P V with P read from TMEM), warp 11 waits for the rings on its behalf,
+//     and warps 2-5 and 6-9 run the online softmax of one query tile each on S
+//     rows straight from TMEM (one thread per row), write P back to TMEM as bf16
+//     over S, rescale O only when the running maximum grew by more than 2^8, and
+//     finally normalise O.  Scores are kept in the log2 domain (scale folded with
+//     log2 e) and exponentiated with ex2.approx.  Rotate-on-load has 16 warps
+//     (see attn_body).
 //  2. combine_kernel (only when the key range of a tile is split over several
 //     CTAs): log-sum-exp merge of the per-split partials (O, m, l), one warp
 //     per query row.
@@ -311,7 +313,7 @@ __device__ __forceinline__ void attn_body(const CUtensorMap &tm_q, const CUtenso
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   // Warp roles: 0 K producer, 1 MMA issuer, then either 2-9 softmax and 10 V
-  // producer, or (rotate-on-load) 2 V producer, 3 idle, 4-11 softmax, 12-15
+  // producer and 11 ring, or (rotate-on-load) 2 V producer, 3 ring, 4-11 softmax, 12-15
   // rotators.
   constexpr int W_V = kFused ? 2 : kWarpV;
   constexpr int W_SM = kFused ? 4 : 2;  // first softmax warp
